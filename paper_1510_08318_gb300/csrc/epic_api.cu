@@ -475,11 +475,12 @@ namespace {
 std::mutex g_fx_lag_mu;
 constexpr int64_t kMaxFxLagEntries = 1LL << 27;   // 2 GB of device tables at most
 
-// The FX route's antenna-pair kernels of every ordered pair (autocorrelations included),
+// The FX route's antenna-pair kernels (autocorrelations included),
 // B_ab(d) = sum over mapping entries e of a and f of b with g_e - g_f = d of w_e conj(w_f)
 // (Eq. "e-field-conv": the cross-correlation of the two sampled footprints), summed per pair in
-// float64 and grouped by wrapped lag cell d into a CSR, uploaded to the plan.  Built once, by the
-// first epic_fx_image call.
+// float64 and grouped by wrapped lag cell d into a CSR, uploaded to the plan.  One order of each
+// pair only: the other order's share of the image is folded into the visibilities (xeng.cu).
+// Built once, by the first epic_fx_image call.
 epic_status build_fx_lag_table(const epic_plan* p) {
     const int A = p->n_ant, NP = p->n_pad, MSK = NP - 1;
     int lg = 0;
@@ -494,6 +495,8 @@ epic_status build_fx_lag_table(const epic_plan* p) {
             y0[a] = std::min(y0[a], gy); y1[a] = std::max(y1[a], gy);
             x0[a] = std::min(x0[a], gx); x1[a] = std::max(x1[a], gx);
         }
+    // entries of the ordered-pair table (both orders of every pair): the documented limit counts
+    // these; the folded table below holds about half of them
     int64_t bound = 0;
     for (int a = 0; a < A; ++a)
         for (int b = 0; b < A; ++b)
@@ -507,19 +510,22 @@ epic_status build_fx_lag_table(const epic_plan* p) {
                          (long long)A * A * p->n_chan * p->n_pol);
     std::vector<int> lag, pair;
     std::vector<float2> w;
-    lag.reserve((size_t)bound);
-    pair.reserve((size_t)bound);
-    w.reserve((size_t)bound);
+    lag.reserve((size_t)bound / 2 + A);
+    pair.reserve((size_t)bound / 2 + A);
+    w.reserve((size_t)bound / 2 + A);
     std::vector<std::complex<double>> win;
     auto weight = [&](int e) {
         float re;
         std::memcpy(&re, &ent[e].x, sizeof(float));
         return std::complex<double>(re, cw ? p->fx_wim_h[e] : 0.0);
     };
-    for (int a = 0; a < A; ++a) {
-        if (y1[a] < 0) continue;
-        for (int b = 0; b < A; ++b) {
-            if (y1[b] < 0) continue;
+    // one order of every unordered pair (fx_pair_swapped says which), numbered as the fold stores them
+    int q = -1;
+    for (int i0 = 0; i0 < A; ++i0) {
+        for (int j0 = i0; j0 < A; ++j0) {
+            ++q;
+            const int a = epic::fx_pair_swapped(i0, j0) ? j0 : i0, b = a == i0 ? j0 : i0;
+            if (y1[a] < 0 || y1[b] < 0) continue;
             const int dy0 = y0[a] - y1[b], dx0 = x0[a] - x1[b];
             const int H = y1[a] - y0[a] + y1[b] - y0[b] + 1, W = x1[a] - x0[a] + x1[b] - x0[b] + 1;
             win.assign((size_t)H * W, std::complex<double>(0.0, 0.0));
@@ -536,7 +542,7 @@ epic_status build_fx_lag_table(const epic_plan* p) {
                     const std::complex<double> v = win[(size_t)i * W + j];
                     if (v == std::complex<double>(0.0, 0.0)) continue;
                     lag.push_back((((dy0 + i) & MSK) << lg) | ((dx0 + j) & MSK));
-                    pair.push_back(a * A + b);
+                    pair.push_back(q);
                     w.push_back(make_float2(float(v.real()), float(v.imag())));
                 }
         }
@@ -556,7 +562,7 @@ epic_status build_fx_lag_table(const epic_plan* p) {
     }
     cudaError_t e;
     if ((e = upload(&p->fx_lag_ptr, lptr)) != cudaSuccess || (e = upload(&p->fx_lag_ent, sent)) != cudaSuccess ||
-        (e = cudaMalloc(&p->fx_vis_t, (size_t)A * A * cp * sizeof(float2))) != cudaSuccess ||
+        (e = cudaMalloc(&p->fx_vis_t, (size_t)A * (A + 1) / 2 * cp * sizeof(float2))) != cudaSuccess ||
         (e = cudaMalloc(&p->fx_u, (size_t)cp * NP * NP * sizeof(float2))) != cudaSuccess) {
         cudaFree(p->fx_lag_ptr);
         cudaFree(p->fx_lag_ent);

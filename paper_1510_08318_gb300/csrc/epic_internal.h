@@ -103,11 +103,15 @@ struct FxArgs {
     const float2* vis;         // [CP][A][A]
     int n_cp, n_ant;
     const int* lag_ptr;        // [N_p^2 + 1] CSR of the antenna-pair kernels by wrapped lag cell
-    const int4* lag_ent;       // {B_ab(d) re bits, im bits, (a * A + b) * CP, 0} of each entry
-    float2* vis_t;             // scratch [A * A][CP]: the visibilities pair-major
+    const int4* lag_ent;       // {B_ab(d) re bits, im bits, pair * CP, 0} of each entry
+    float2* vis_t;             // scratch [A (A + 1) / 2][CP]: the folded visibilities pair-major
     float2* u;                 // scratch [CP][N_p][N_p]: the lag planes
     float* image;              // [CP][N_p][N_p]
 };
+// Which order of the unordered pair i <= j the lag table and the folded visibilities use: (i, j), or
+// (j, i) where this is true.  Alternating orders spread the lags of an array whose antennas are
+// listed in some spatial order over the whole lag plane instead of one half of it.
+__host__ __device__ inline bool fx_pair_swapped(int i, int j) { return ((i + j) & 1) != 0; }
 cudaError_t launch_fx_image(int n_pad, const FxArgs& a, cudaStream_t st);
 cudaError_t launch_xeng(int vdt, const XengArgs& a, int n_sm, cudaStream_t st);
 

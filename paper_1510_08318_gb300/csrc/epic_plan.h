@@ -27,8 +27,8 @@ struct epic_plan {
     std::vector<int2> fx_ent_h;
     std::vector<float> fx_wim_h;
     // The FX route's antenna-pair kernels B_ab(d) grouped by lag cell d (CSR over the N_p^2 wrapped
-    // lags: {weight re bits, im bits, (a * A + b) * C * P, 0}) and the imaging scratch (the
-    // visibilities pair-major, the lag planes), built by the first epic_fx_image call
+    // lags: {weight re bits, im bits, pair * C * P, 0}, one order of each pair) and the imaging
+    // scratch (the folded visibilities pair-major, the lag planes), built by the first epic_fx_image call
     mutable int* fx_lag_ptr = nullptr;
     mutable int4* fx_lag_ent = nullptr;
     mutable float2* fx_vis_t = nullptr;

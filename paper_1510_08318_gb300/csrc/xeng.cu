@@ -450,9 +450,12 @@ __global__ void __launch_bounds__(NT, 1) xeng_kernel(const XengArgs a) {
 // ---- the FX route's imaging of an integration's visibilities (Eq. "dirty-image-FX") ----
 //   U(d) = sum_{a, b} V_ab B_ab(d),  B_ab(d) = sum_g M[g, a] conj(M[g - d, b]),
 //   I(k) = Re sum_d U(d) exp(+2 pi i d.k / N_p)  (image pixel order, k = 0 at the centre).
-// Three launches.  (1) The visibilities are transposed to pair-major order with the (channel,
-// pol) index innermost, so that the values of one pair for consecutive (channel, pol) are
-// contiguous.  (2) The lag planes are gathered from the plan's table of the antenna-pair kernels
+// Since B_ba(d) = conj(B_ab(-d)), the two orders of a pair add Re(S V_ab) + Re(conj(S) V_ba) to a
+// pixel, S = sum_d B_ab(d) exp(+2 pi i d.k / N_p): one order with V_ab + conj(V_ba) gives the same
+// image from half the table, for any visibilities (they need not be Hermitian).
+// Three launches.  (1) The two orders of every pair are folded into one and written in pair-major
+// order with the (channel, pol) index innermost, so that the values of one pair for consecutive
+// (channel, pol) are contiguous.  (2) The lag planes are gathered from the plan's table of the antenna-pair kernels
 // grouped by lag cell (B_ab(d) summed over the mapping entries of a and b once, on the host): a
 // warp takes one lag cell for a group of G (channel, pol) planes, its lanes G planes x 32 / G
 // entries, so that each entry's visibilities are one coalesced load for the G planes (no
@@ -462,24 +465,48 @@ __global__ void __launch_bounds__(NT, 1) xeng_kernel(const XengArgs a) {
 // register DFTs, a twiddle, S1-point register DFTs across the line's threads), rows then
 // columns, the real part written as the image.
 
-// (1) vis [CP][P2] -> vis_t [P2][CP] through 32 x 32 shared-memory tiles
-__global__ void __launch_bounds__(256) fx_transpose_kernel(const float2* __restrict__ vis, int n_cp, long long n_pair,
-                                                           float2* __restrict__ vis_t) {
-    __shared__ float2 tile[32][33];
-    const long long p0 = (long long)blockIdx.x * 32;
-    const int c0 = blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-#pragma unroll
-    for (int j = 0; j < 32; j += 8) {
-        const int c = c0 + ty + j;
-        const long long p = p0 + tx;
-        if (c < n_cp && p < n_pair) tile[ty + j][tx] = __ldg(vis + (size_t)c * n_pair + p);
+// (1) The fold: for i < j the pair's two orders become one, W = V_ij + conj(V_ji) (or its conjugate
+// where the table uses the order (j, i)); W = V_ii on the diagonal.  vis [CP][A][A] -> vis_t
+// [pair][CP], pair = the packed index of i <= j.  A block takes FXT_A rows i and 32 columns j for 32
+// planes: V_ij is read 32 columns (256 bytes) at a time, V_ji 4 columns (one 32-byte sector) of 32
+// rows, and 32 planes of a pair are written as 256 bytes.  HBM-bound: every visibility is read once.
+constexpr int FXT_A = 4;
+constexpr int FXT_J = 33, FXT_I = 32 * FXT_J + 4;   // strides of the tile (float2): no bank conflicts
+
+__global__ void __launch_bounds__(256) fx_fold_kernel(const float2* __restrict__ vis, int n_cp, int A,
+                                                      float2* __restrict__ vis_t) {
+    __shared__ float2 tile[FXT_A * FXT_I];
+    const int j0 = blockIdx.x * 32, i0 = blockIdx.y * FXT_A, c0 = blockIdx.z * 32;
+    if (j0 + 31 < i0) return;                       // below the diagonal
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const size_t plane = (size_t)A * A;
+    // V_ij: a warp reads the 32 columns of one (row, plane)
+#pragma unroll 4
+    for (int q = warp; q < FXT_A * 32; q += 8) {
+        const int i = i0 + q / 32, c = c0 + q % 32, j = j0 + lane;
+        if (c < n_cp && i < A && j < A && j >= i)
+            tile[(q / 32) * FXT_I + lane * FXT_J + q % 32] = __ldg(vis + (size_t)c * plane + (size_t)i * A + j);
     }
     __syncthreads();
-#pragma unroll
-    for (int j = 0; j < 32; j += 8) {
-        const long long p = p0 + ty + j;
-        const int c = c0 + tx;
-        if (c < n_cp && p < n_pair) vis_t[(size_t)p * n_cp + c] = tile[tx][ty + j];
+    // V_ji: 4 columns i of 8 rows j
+#pragma unroll 4
+    for (int q = warp; q < 4 * 32; q += 8) {
+        const int ii = lane & 3, jj = (q / 32) * 8 + (lane >> 2), cc = q % 32;
+        const int i = i0 + ii, j = j0 + jj, c = c0 + cc;
+        if (c < n_cp && j < A && j > i) {
+            const float2 u = __ldg(vis + (size_t)c * plane + (size_t)j * A + i);
+            float2* t = tile + ii * FXT_I + jj * FXT_J + cc;
+            const float2 v = make_float2(t->x + u.x, t->y - u.y);
+            *t = fx_pair_swapped(i, j) ? make_float2(v.x, -v.y) : v;
+        }
+    }
+    __syncthreads();
+    for (int q = warp; q < FXT_A * 32; q += 8) {
+        const int i = i0 + q / 32, j = j0 + q % 32, c = c0 + lane;
+        if (c < n_cp && i < A && j < A && j >= i) {
+            const size_t pair = (size_t)i * A - (size_t)i * (i - 1) / 2 + (j - i);
+            vis_t[pair * n_cp + c] = tile[(q / 32) * FXT_I + (q % 32) * FXT_J + lane];
+        }
     }
 }
 
@@ -489,34 +516,52 @@ __global__ void __launch_bounds__(256) fx_transpose_kernel(const float2* __restr
 // G planes; the CTAs of one tile (all groups) are adjacent in launch order so that they share
 // the tile's table entries in L2.  A warp takes whole lag cells.  It reads the entries of a cell
 // 32 at a time with one coalesced load into its own shared-memory slots (slots past the cell's
-// end hold zero weights at offset 0; the next 32 entries are loaded while these are used).
-// V4 (an even number of planes, G = 64): lane c takes planes 2c, 2c + 1 of the group with one
-// 16-byte load per entry, every lane every entry, 8 entries in flight.  Otherwise lane =
-// e * G + c (plane c, G <= 32) takes entries e, e + E, ... of the 32 (E = 32 / G) with 8-byte
-// loads, up to 16 in flight, and the sum over a cell's entries ends with a shuffle over e.
-constexpr int FXG_NT = 256;
+// end hold zero weights at offset 0; the next 32 entries are loaded while these are used).  An
+// entry takes G / W lanes of W planes each, E = 32 W / G entries side by side, and the sum over a
+// cell's entries ends with a shuffle.  V4 (an even number of planes): W = 2, one 16-byte load per
+// lane and entry; else W = 1 with 8-byte loads.
+//
+// What bounds it: the visibilities' way from L2 to L1 (each pair is used by up to 81 lag cells), then
+// L1 wavefronts, and for few planes the tiles around lag 0, which hold several times the mean number
+// of entries.  Measured on a 256-antenna layout (N_p = 128; all three launches): 965 us at 128 planes
+// with both orders of every pair gathered, G = 64 and 8-warp CTAs; 538 with one order; 412 with
+// G = 16 (a tile's pairs then mostly stay in L1); 286 with the tiles ordered by their distance from
+// lag 0; 229 with one 32-warp CTA per SM, which shortens the longest tiles fourfold (64 registers,
+// 4 loads in flight per lane).  The width G: see launch_fx_image_t.
+constexpr int FXG_NT = 1024;
 
 template <int G, bool V4>
-__global__ void __launch_bounds__(FXG_NT, V4 ? 2 : 3) fx_gather_kernel(const FxArgs a, int np) {
-    static_assert(V4 ? G == 64 : G <= 32, "group width");
-    constexpr int E = V4 ? 1 : 32 / G;                                   // entry slots per step
-    constexpr int U = V4 ? 8 : ((16 * E <= 32) ? 16 : 32 / E);           // entries per lane in flight
+__global__ void __launch_bounds__(FXG_NT, 1) fx_gather_kernel(const FxArgs a, int np) {
+    static_assert(G <= 32 && (!V4 || G >= 2), "group width");
+    constexpr int W = V4 ? 2 : 1;                                        // planes per lane
+    constexpr int LPE = G / W;                                           // lanes per entry
+    constexpr int E = 32 / LPE;                                          // entry slots per step
+    constexpr int U0 = V4 ? 4 : 16;
+    constexpr int U = (U0 * E <= 32) ? U0 : 32 / E;                      // entries per lane in flight
     static_assert(U * E <= 32 && 32 % (U * E) == 0, "steps");
     __shared__ int4 sent[FXG_NT / 32][32];
     const int CP = a.n_cp, n_groups = (CP + G - 1) / G;
     const int tiles_x = np / 8;
     const int tile = blockIdx.x / n_groups, gi = blockIdx.x - tile * n_groups;
-    const int ty0 = 8 * (tile / tiles_x), tx0 = 8 * (tile % tiles_x);
+    // tiles in the order of their distance from lag 0 (the wrapped corners), where most pairs lie, so
+    // that the longest blocks start first: the tile number's even and odd bits are the positions
+    // along x and y, position p the p-th nearest tile row to lag 0
+    int ix = 0, iy = 0;
+    for (int bit = 0; (1 << bit) < tiles_x; ++bit) {
+        ix |= ((tile >> (2 * bit)) & 1) << bit;
+        iy |= ((tile >> (2 * bit + 1)) & 1) << bit;
+    }
+    const int ty0 = 8 * ((iy & 1) ? tiles_x - 1 - iy / 2 : iy / 2), tx0 = 8 * ((ix & 1) ? tiles_x - 1 - ix / 2 : ix / 2);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int e = V4 ? 0 : lane / G;
-    const int cp = V4 ? gi * G + 2 * lane : gi * G + lane % G;          // first plane of the lane
-    const bool valid = cp < CP;
+    const int e = lane / LPE;
+    const int cp = gi * G + W * (lane % LPE);                            // first plane of the lane
+    const bool valid = cp < CP;                                          // (V4: CP is even)
     const float2* Vt = a.vis_t + (valid ? cp : 0);
     int4* sw = sent[warp];
     for (int j = warp; j < 64; j += FXG_NT / 32) {
         const int d = (ty0 + (j >> 3)) * np + tx0 + (j & 7);
         const int p0 = __ldg(a.lag_ptr + d), p1 = __ldg(a.lag_ptr + d + 1);
-        float2 acc = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
+        float2 acc[W] = {};
         int4 nxt = p0 + lane < p1 ? __ldg(a.lag_ent + p0 + lane) : make_int4(0, 0, 0, 0);
         for (int q0 = p0; q0 < p1; q0 += 32) {
             const int nb = min(32, p1 - q0);
@@ -525,51 +570,37 @@ __global__ void __launch_bounds__(FXG_NT, V4 ? 2 : 3) fx_gather_kernel(const FxA
             __syncwarp();
             nxt = q0 + 32 + lane < p1 ? __ldg(a.lag_ent + q0 + 32 + lane) : make_int4(0, 0, 0, 0);
             for (int k = 0; k < nb; k += U * E) {
-                if constexpr (V4) {
-                    float4 v[U];
-                    float2 w[U];
+                float2 v[U][W], w[U];
 #pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const int4 en = sw[k + u];
-                        w[u] = make_float2(__int_as_float(en.x), __int_as_float(en.y));
-                        v[u] = __ldg(reinterpret_cast<const float4*>(Vt + en.z));
-                    }
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        acc.x = fmaf(v[u].x, w[u].x, fmaf(-v[u].y, w[u].y, acc.x));
-                        acc.y = fmaf(v[u].x, w[u].y, fmaf(v[u].y, w[u].x, acc.y));
-                        acc1.x = fmaf(v[u].z, w[u].x, fmaf(-v[u].w, w[u].y, acc1.x));
-                        acc1.y = fmaf(v[u].z, w[u].y, fmaf(v[u].w, w[u].x, acc1.y));
-                    }
-                } else {
-                    float2 v[U], w[U];
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const int4 en = sw[k + u * E + e];
-                        w[u] = make_float2(__int_as_float(en.x), __int_as_float(en.y));
-                        v[u] = __ldg(Vt + en.z);
-                    }
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        acc.x = fmaf(v[u].x, w[u].x, fmaf(-v[u].y, w[u].y, acc.x));
-                        acc.y = fmaf(v[u].x, w[u].y, fmaf(v[u].y, w[u].x, acc.y));
+                for (int u = 0; u < U; ++u) {
+                    const int4 en = sw[k + u * E + e];
+                    w[u] = make_float2(__int_as_float(en.x), __int_as_float(en.y));
+                    if constexpr (V4) {
+                        const float4 f = __ldg(reinterpret_cast<const float4*>(Vt + en.z));
+                        v[u][0] = make_float2(f.x, f.y);
+                        v[u][1] = make_float2(f.z, f.w);
+                    } else {
+                        v[u][0] = __ldg(Vt + en.z);
                     }
                 }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int i = 0; i < W; ++i) {
+                        acc[i].x = fmaf(v[u][i].x, w[u].x, fmaf(-v[u][i].y, w[u].y, acc[i].x));
+                        acc[i].y = fmaf(v[u][i].x, w[u].y, fmaf(v[u][i].y, w[u].x, acc[i].y));
+                    }
             }
         }
         const size_t npix = (size_t)np * np;
-        if constexpr (V4) {
-            if (valid) {
-                a.u[(size_t)cp * npix + d] = acc;
-                a.u[(size_t)(cp + 1) * npix + d] = acc1;
-            }
-        } else {
 #pragma unroll
-            for (int o = 16; o >= G; o >>= 1) {
-                acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-                acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+        for (int i = 0; i < W; ++i) {
+#pragma unroll
+            for (int o = 16; o >= LPE; o >>= 1) {
+                acc[i].x += __shfl_xor_sync(0xffffffffu, acc[i].x, o);
+                acc[i].y += __shfl_xor_sync(0xffffffffu, acc[i].y, o);
             }
-            if (e == 0 && valid) a.u[(size_t)cp * npix + d] = acc;
+            if (e == 0 && valid) a.u[(size_t)(cp + i) * npix + d] = acc[i];
         }
     }
 }
@@ -692,26 +723,29 @@ __global__ void __launch_bounds__(FxDft<NP>::NT) fx_dft_kernel(const float2* __r
 
 template <int NP>
 cudaError_t launch_fx_image_t(const FxArgs& a, cudaStream_t st) {
-    const long long n_pair = (long long)a.n_ant * a.n_ant;
-    fx_transpose_kernel<<<dim3((unsigned)((n_pair + 31) / 32), (unsigned)((a.n_cp + 31) / 32)), 256, 0, st>>>(
-        a.vis, a.n_cp, n_pair, a.vis_t);
+    fx_fold_kernel<<<dim3((unsigned)((a.n_ant + 31) / 32), (unsigned)((a.n_ant + FXT_A - 1) / FXT_A),
+                          (unsigned)((a.n_cp + 31) / 32)), 256, 0, st>>>(a.vis, a.n_cp, a.n_ant, a.vis_t);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const long long tiles = (NP / 8) * (NP / 8);
-    if (a.n_cp >= 64 && a.n_cp % 2 == 0) {
-        fx_gather_kernel<64, true><<<(unsigned)(tiles * ((a.n_cp + 63) / 64)), FXG_NT, 0, st>>>(a, NP);
-    } else {
-        int g = 1;
-        while (g < 32 && g < a.n_cp) g *= 2;
-        const unsigned blocks = (unsigned)(tiles * ((a.n_cp + g - 1) / g));
-        switch (g) {
-            case 1: fx_gather_kernel<1, false><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
-            case 2: fx_gather_kernel<2, false><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
-            case 4: fx_gather_kernel<4, false><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
-            case 8: fx_gather_kernel<8, false><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
-            case 16: fx_gather_kernel<16, false><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
-            default: fx_gather_kernel<32, false><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
-        }
+    // Planes per group: narrow groups keep more of a tile's pairs in L1 and give more CTAs, wide ones
+    // read each table entry and its row of visibilities fewer times.  Measured (us; 256 antennas,
+    // N_p = 128) with 2, 4, 8, 16, 32 planes per group: 4 planes 64, 68, 78, -, -; 8 planes 88, 72, 81,
+    // 107, -; 16 planes 167, 99, 89, 108, 171; 32 planes 310, 170, 107, 109, 181; 64 planes 616, 333,
+    // 198, 141, 189; 128 planes -, -, 367, 252, 229.
+    const int g = a.n_cp >= 96 ? 32 : a.n_cp >= 40 ? 16 : a.n_cp >= 12 ? 8 : a.n_cp >= 6 ? 4 : a.n_cp >= 2 ? 2 : 1;
+    const unsigned blocks = (unsigned)((NP / 8) * (NP / 8) * (long long)((a.n_cp + g - 1) / g));
+    switch (2 * g + (a.n_cp % 2 == 0 ? 1 : 0)) {
+        case 2: fx_gather_kernel<1, false><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
+        case 4: fx_gather_kernel<2, false><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
+        case 5: fx_gather_kernel<2, true><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
+        case 8: fx_gather_kernel<4, false><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
+        case 9: fx_gather_kernel<4, true><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
+        case 16: fx_gather_kernel<8, false><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
+        case 17: fx_gather_kernel<8, true><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
+        case 32: fx_gather_kernel<16, false><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
+        case 33: fx_gather_kernel<16, true><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
+        case 64: fx_gather_kernel<32, false><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
+        default: fx_gather_kernel<32, true><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     using D = FxDft<NP>;

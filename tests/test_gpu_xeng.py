@@ -231,3 +231,26 @@ def test_longest_integration_reaches_2_to_24(epic):
     with pytest.raises(epic.EpicError) as e:
         plan.correlate(torch.full((T + 1, 1, 1, 16), 0x88, dtype=torch.uint8, device="cuda"))
     assert e.value.status == epic.EPIC_EUNSUPPORTED
+
+
+@pytest.mark.parametrize("n_cp, n_ant", [(4, 5), (7, 33), (8, 34), (13, 9), (16, 64), (97, 6), (128, 37)])
+def test_gpu_fx_image_folded_pairs(epic, n_cp, n_ant):
+    """The fold of a pair's two orders and every width of the gather's plane groups (2, 4, 8, 16, 32,
+    even and odd plane counts), on visibilities that are not Hermitian and antenna counts that leave
+    ragged fold tiles: against the pairwise sum Re sum_ab V_ab K_a conj(K_b) in float64.  The bound:
+    products and sums of n_ant^2 x 9 FP32 terms of random sign, 1e-5 of the plane's norm."""
+    rng = np.random.default_rng(n_cp)
+    n_grid, n_pad = 14, 32
+    pos = np.sort(rng.uniform(2.0, n_grid - 3.0, (n_ant, 2)), axis=0)
+    ptr, dxdy, w = synth.pack_kernels([synth.kernel_square(2.5, 1.0)] * n_ant)
+    w = w * np.exp(1j * rng.uniform(0, 2 * np.pi, w.shape))
+    plan = epic.Plan(pos, ptr, dxdy, w, 1.0, np.zeros(2), n_grid, n_pad, n_cp, 1, "c64")
+    vis = (rng.standard_normal((n_cp, 1, n_ant, n_ant)) + 1j * rng.standard_normal((n_cp, 1, n_ant, n_ant)))
+    img = plan.fx_image(torch.from_numpy(vis.astype(np.complex64)).cuda()).cpu().numpy()
+    M = moff.map_antennas(pos, ptr, dxdy, w, 1.0, np.zeros(2), n_grid)
+    K = np.stack([np.fft.fftshift(np.fft.ifft2(np.asarray(M[:, a].todense() if hasattr(M, "todense") else M[:, a])
+                                               .reshape(n_grid, n_grid), s=(n_pad, n_pad), norm="forward"))
+                  for a in range(n_ant)]).reshape(n_ant, -1)
+    for c in range(n_cp):
+        want = (K * (vis[c, 0].astype(np.complex64).astype(np.complex128) @ K.conj())).sum(0).real.reshape(n_pad, n_pad)
+        assert np.linalg.norm(img[c, 0] - want) < 1e-5 * np.linalg.norm(want), c
