@@ -66,6 +66,11 @@ void free_plan(epic_plan* p) {
     cudaFree(p->twiddle);
     cudaFree(p->lag_tab);
     cudaFree(p->dg_tab);
+    cudaFree(p->dp_lane);
+    cudaFree(p->dp_slot);
+    cudaFree(p->dp_w);
+    cudaFree(p->dp_wim);
+    cudaFree(p->dp_ant);
     cudaFree(p->dg_lane);
     cudaFree(p->dg_base);
     cudaFree(p->dg_wre);
@@ -325,14 +330,17 @@ epic_status epic_create(epic_plan** plan, int n_ant, const double* pos_xy, const
     std::vector<int> dbase;
     std::vector<float> dwre, dwim;
     std::vector<uint16_t> dant;
-    const bool dg_ok = (n_pad == 128 && epic::dftgemm_gather_tables(cptr, cent, cwim, dlane, dbase, dwre, dwim, dant)) ||
-                       (n_pad == 256 &&
-                        epic::dftgemm_gather_tables_ng(128, epic::kDg256GridWarps, cptr, cent, cwim, dlane, dbase,
-                                                       dwre, dwim, dant));
+    std::vector<uint32_t> plane;
+    std::vector<int2> pslot;
+    std::vector<float2> pw, pwim;
+    std::vector<uint16_t> pant;
+    const bool dp_ok = n_pad == 128 && epic::dftgemm_pair_tables(cptr, cent, cwim, plane, pslot, pw, pwim, pant);
+    const bool dg_ok = n_pad == 256 && epic::dftgemm_gather_tables_ng(128, epic::kDg256GridWarps, cptr, cent, cwim, dlane,
+                                                                      dbase, dwre, dwim, dant);
     // N_p = 256 with real weights: the same entries packed one word each for the FP16-gridding
     // form, (FP16 weight, rounded to nearest) << 16 | antenna
     std::vector<uint32_t> dwpk;
-    if (dg_ok && n_pad == 256 && !complex_w) {
+    if (dg_ok && !complex_w) {
         dwpk.resize(dwre.size());
         for (size_t q = 0; q < dwre.size(); ++q)
             dwpk[q] = ((uint32_t)__half_as_ushort(__float2half_rn(dwre[q])) << 16) | (uint32_t)dant[q];
@@ -450,6 +458,9 @@ epic_status epic_create(epic_plan** plan, int n_ant, const double* pos_xy, const
         (SL > 0 && ((e = upload(&p->wlane, wlane)) != cudaSuccess || (e = upload(&p->wbase, wbase)) != cudaSuccess ||
                     (e = upload(&p->went, went)) != cudaSuccess ||
                     (complex_w && (e = upload(&p->wwim, wwim)) != cudaSuccess))) ||
+        (dp_ok && ((e = upload(&p->dp_lane, plane)) != cudaSuccess || (e = upload(&p->dp_slot, pslot)) != cudaSuccess ||
+                   (e = upload(&p->dp_w, pw)) != cudaSuccess || (e = upload(&p->dp_ant, pant)) != cudaSuccess ||
+                   (complex_w && (e = upload(&p->dp_wim, pwim)) != cudaSuccess))) ||
         (dg_ok && ((e = upload(&p->dg_lane, dlane)) != cudaSuccess || (e = upload(&p->dg_base, dbase)) != cudaSuccess ||
                    (e = upload(&p->dg_wre, dwre)) != cudaSuccess || (e = upload(&p->dg_ant, dant)) != cudaSuccess ||
                    (complex_w && (e = upload(&p->dg_wim, dwim)) != cudaSuccess) ||
@@ -458,6 +469,7 @@ epic_status epic_create(epic_plan** plan, int n_ant, const double* pos_xy, const
         return e == cudaErrorMemoryAllocation ? epic_fail(EPIC_ENOMEM, "plan tables: %s", cudaGetErrorString(e))
                                               : epic_cuda_fail(e, "plan upload");
     }
+    p->dp_n = (int)pant.size();
     p->fx_ptr_h = fxptr;
     p->fx_ent_h = fxent;
     p->fx_wim_h = fxwim;
@@ -650,7 +662,7 @@ epic_status epic_set_transform(epic_plan* plan, int xform) {
     if (xform == EPIC_XFORM_DFTGEMM_FP16_GRID && plan->n_pad != 256)
         return epic_fail(EPIC_EUNSUPPORTED, "the FP16-gridding tensor-core form exists for n_pad 256 only (plan: %d)",
                          plan->n_pad);
-    if (!plan->dg_lane)
+    if (plan->n_pad == 128 ? !plan->dp_lane : !plan->dg_lane)
         return epic_fail(EPIC_EUNSUPPORTED, "a pair of grid cells has more than 65535 mapping entries, or more than "
                                             "65536 antennas");
     if (xform == EPIC_XFORM_DFTGEMM_FP16_GRID && !plan->dg_wim && !plan->dg_wpk)
@@ -733,12 +745,16 @@ epic_status epic_image(const epic_plan* plan, const void* volt, int n_time, cons
     epic_status s;
     if (plan->xform == EPIC_XFORM_DFTGEMM || plan->xform == EPIC_XFORM_DFTGEMM_FP16 ||
         plan->xform == EPIC_XFORM_DFTGEMM_FP16_GRID) {
-        const epic::DgGather g{plan->dg_lane, plan->dg_base, plan->dg_wre, plan->dg_wim, plan->dg_ant, (int)plan->nnz,
-                               plan->dg_wpk};
-        e = plan->n_pad == 128 ? epic::launch_dftgemm(plan->vdt, a, plan->dg_tab, g, plan->n_sm, st, false,
-                                                      plan->xform == EPIC_XFORM_DFTGEMM_FP16)
-                               : epic::launch_dftgemm256(plan->vdt, a, plan->dg_tab, g, plan->n_sm, st,
-                                                         plan->xform == EPIC_XFORM_DFTGEMM_FP16_GRID);
+        if (plan->n_pad == 128) {
+            const epic::DgPairGather g{plan->dp_lane, plan->dp_slot, plan->dp_w, plan->dp_wim, plan->dp_ant, plan->dp_n};
+            e = epic::launch_dftgemm(plan->vdt, a, plan->dg_tab, g, plan->n_sm, st, false,
+                                     plan->xform == EPIC_XFORM_DFTGEMM_FP16);
+        } else {
+            const epic::DgGather g{plan->dg_lane, plan->dg_base, plan->dg_wre, plan->dg_wim, plan->dg_ant,
+                                   (int)plan->nnz, plan->dg_wpk};
+            e = epic::launch_dftgemm256(plan->vdt, a, plan->dg_tab, g, plan->n_sm, st,
+                                        plan->xform == EPIC_XFORM_DFTGEMM_FP16_GRID);
+        }
         s = e == cudaSuccess ? EPIC_OK : epic_cuda_fail(e, "tensor-core imaging kernel launch");
     } else if (plan->xform == EPIC_XFORM_FFT_TWOPASS) {
         epic::SegList L;
@@ -854,7 +870,7 @@ epic_status epic_image_xpol(const epic_plan* plan, const void* volt, int n_time,
     a.n_items = (long long)a.n_cp * n_time;
     epic_status s;
     if (dg) {
-        const epic::DgGather g{plan->dg_lane, plan->dg_base, plan->dg_wre, plan->dg_wim, plan->dg_ant, (int)plan->nnz};
+        const epic::DgPairGather g{plan->dp_lane, plan->dp_slot, plan->dp_w, plan->dp_wim, plan->dp_ant, plan->dp_n};
         e = epic::launch_dftgemm(plan->vdt, a, plan->dg_tab, g, plan->n_sm, st, true);
         s = e == cudaSuccess ? EPIC_OK : epic_cuda_fail(e, "tensor-core cross-polarisation kernel launch");
     } else {

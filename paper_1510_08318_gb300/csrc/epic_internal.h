@@ -155,14 +155,23 @@ int grid_rows_per_block(int n_pad);   // rows of the N_g grid each CTA of a clus
 int fwd_interleave_lanes(int n_pad);  // S of the warp-interleaved mapping, 0 if the size does not use it
 int exchange_row_stride(int n_pad);   // row stride (float2) of the kernels' exchange buffer
 
-// Tensor-core DFT form of the forward kernel, N_p = 128 (moff_dftgemm.cu).
-// Its gridding walks the 2048 cell pairs (x, y), (x, y + 1), y even, of the 64 x 64 grid in 64
-// slots of 32 pairs ranked by entry count (most first), lanes of a slot in rank order; step k
-// of a slot holds the k-th entry of every lane whose pair has more than k entries (the entries
-// of cell y in cell-major order, then those of cell y + 1).
+// Gathers of the tensor-core DFT forms: the cell pairs (x, y), (x, y + 1), y even, of the N_g x N_g
+// grid in slots of 32 pairs ranked by entry count (most first), lanes of a slot in rank order.
+// N_p = 128 (moff_dftgemm.cu), 64 slots: an entry is an antenna with its weights on both cells; step k
+// of a slot is the 32 entries from its first + 32 k on, zero weights where a lane's list has ended.
+struct DgPairGather {
+    const uint32_t* lane;  // [66][32] E^T table offset of (x, y) | (x + y) << 16, by slot position
+    const int2* slot;      // [66] {first entry, steps} of each position's slot; -1 steps: holds none
+    const float2* w;       // entry weights on (x, y) and (x, y + 1), real parts
+    const float2* wim;     // imaginary parts, or nullptr when every weight is real
+    const uint16_t* ant;   // entry antennas
+    int n_ent;             // number of entries
+};
+// N_p = 256 (moff_dftgemm256.cu): an entry is one cell's (the entries of cell y, then those of cell
+// y + 1); step k of a slot holds the k-th entry of every lane whose pair has more than k entries.
 struct DgGather {
-    const int2* lane;      // [64][32] {entries of cell y | (entries of the pair) << 16, E^T table offset of (x, y)}
-    const int* base;       // [64] first entry of each slot
+    const int2* lane;      // [slots][32] {entries of cell y | (entries of the pair) << 16, E^T table offset of (x, y)}
+    const int* base;       // [slots] first entry of each slot, -1 where a warp's position holds none
     const float* wre;      // entry weights, real parts
     const float* wim;      // entry weights, imaginary parts, or nullptr when every weight is real
     const uint16_t* ant;   // entry antennas
@@ -171,14 +180,18 @@ struct DgGather {
     // (read by the FP16-gridding form); nullptr otherwise
     const uint32_t* wpk = nullptr;
 };
-// the least a launch needs (tables read through L1); lp: the reduced-precision form (FP16
-// operands and one product per real product)
+// N_p = 128: the size that decides how many antennas the form accepts (a launch needs at most this); lp:
+// the reduced-precision form (FP16 operands and one product per real product)
 size_t dftgemm_smem_bytes(int n_ant, bool xpol = false, bool lp = false);
 void dftgemm_tables(std::vector<uint16_t>& out);
 // false if a pair has more than 65535 entries or an antenna index does not fit 16 bits
 bool dftgemm_gather_tables(const std::vector<int>& cptr, const std::vector<int2>& cent, const std::vector<float>& cwim,
                            std::vector<int2>& lane, std::vector<int>& base, std::vector<float>& wre,
                            std::vector<float>& wim, std::vector<uint16_t>& ant);
+// Slot tables of the N_p = 128 kernel (DgPairGather); false as above.
+bool dftgemm_pair_tables(const std::vector<int>& cptr, const std::vector<int2>& cent, const std::vector<float>& cwim,
+                         std::vector<uint32_t>& lane, std::vector<int2>& slot, std::vector<float2>& w,
+                         std::vector<float2>& wim, std::vector<uint16_t>& ant);
 // The same slot tables for a grid of ng x ng cells (ng = 64 or 128; ng^2 / 64 slots) gridded by
 // n_warps warps, warp w walking the ceil(slots / n_warps) positions from w * that (positions no
 // slot took are empty).  false as above, or for another ng.
@@ -186,7 +199,7 @@ bool dftgemm_gather_tables_ng(int ng, int n_warps, const std::vector<int>& cptr,
                               const std::vector<float>& cwim, std::vector<int2>& lane, std::vector<int>& base,
                               std::vector<float>& wre, std::vector<float>& wim, std::vector<uint16_t>& ant);
 // xpol: the (channel, pol) items are the 4 C virtual pols of dual-pol data, as in the FFT form
-cudaError_t launch_dftgemm(int vdt, const FwdArgs& a, const void* wtab, const DgGather& g, int n_sm, cudaStream_t st,
+cudaError_t launch_dftgemm(int vdt, const FwdArgs& a, const void* wtab, const DgPairGather& g, int n_sm, cudaStream_t st,
                            bool xpol = false, bool lp = false);
 
 // Tensor-core DFT form for N_p = 256 (moff_dftgemm256.cu): two CTAs per image (one per half of

@@ -41,7 +41,13 @@ struct epic_plan {
     float2* lag_tab = nullptr;
     int xform = EPIC_XFORM_FFT;
     uint16_t* dg_tab = nullptr;   // DFT operand tables of the tensor-core form
-    int2* dg_lane = nullptr;      // gridding slot tables of the tensor-core form (N_p = 128)
+    uint32_t* dp_lane = nullptr;  // gridding slot tables of the tensor-core form, N_p = 128 (DgPairGather)
+    int2* dp_slot = nullptr;
+    float2* dp_w = nullptr;
+    float2* dp_wim = nullptr;
+    uint16_t* dp_ant = nullptr;
+    int dp_n = 0;
+    int2* dg_lane = nullptr;      // the same, N_p = 256 (DgGather)
     int* dg_base = nullptr;
     float* dg_wre = nullptr;
     float* dg_wim = nullptr;

@@ -129,29 +129,6 @@ __global__ void __launch_bounds__(TA * Split<C>::R2, (TA * Split<C>::R2 <= 256) 
 // loads, stores, address arithmetic and twiddle loads of a thread serve two antennas.
 struct P2 { unsigned long long re, im; };
 
-__device__ __forceinline__ unsigned long long f2add(unsigned long long a, unsigned long long b) {
-    unsigned long long r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ unsigned long long f2sub(unsigned long long a, unsigned long long b) {
-    unsigned long long r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ unsigned long long f2mul(unsigned long long a, unsigned long long b) {
-    unsigned long long r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-// a * b + c, each lane rounded once
-__device__ __forceinline__ unsigned long long f2fma(unsigned long long a, unsigned long long b, unsigned long long c) {
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ unsigned long long f2dup(float c) { return pack2(make_float2(c, c)); }
-
 // (a - b) * exp(SIGN 2 pi i m / M) for a compile-time rotation; the half and quarter turns cost
 // no multiplies (the swap and the sign go into the subtraction).
 template <int SIGN>
