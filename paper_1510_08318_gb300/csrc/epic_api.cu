@@ -736,9 +736,8 @@ epic_status epic_image(const epic_plan* plan, const void* volt, int n_time, cons
     const size_t npix = (size_t)cp * plan->n_pad * plan->n_pad;
     cudaError_t e;
     if (t_prev == 0) {
-        if ((e = cudaMemsetAsync(accum, 0, npix * sizeof(double), st)) != cudaSuccess) return epic_cuda_fail(e, "memset accum");
-        if (power && (e = cudaMemsetAsync(power, 0, (size_t)cp * plan->n_ant * sizeof(double), st)) != cudaSuccess)
-            return epic_cuda_fail(e, "memset power");
+        e = epic::launch_zero(accum, (long long)npix, power, (long long)cp * plan->n_ant, st);
+        if (e != cudaSuccess) return epic_cuda_fail(e, "zeroing the accumulators");
     }
     const epic::FwdArgs a =
         epic_plan_fwd_args(plan, volt, n_time, reinterpret_cast<const float2*>(gains), accum, power);
@@ -774,11 +773,14 @@ epic_status epic_image(const epic_plan* plan, const void* volt, int n_time, cons
     }
     if (s != EPIC_OK) return s;
     const double inv_t = 1.0 / double(t_prev + n_time);
-    if (image && (e = epic::launch_finalize_image(accum, image, (long long)npix, inv_t, st)) != cudaSuccess)
-        return epic_cuda_fail(e, "image epilogue");
-    if (autocorr && (e = epic::launch_autocorr(power, plan->lag_tab, cp, plan->n_ant, plan->lag_side, plan->n_pad,
-                                               inv_t, autocorr, st)) != cudaSuccess)
-        return epic_cuda_fail(e, "auto-correlation epilogue");
+    if (autocorr) {
+        e = epic::launch_autocorr(power, plan->lag_tab, plan->twiddle, cp, plan->n_ant, plan->lag_side, plan->n_pad, inv_t, autocorr,
+                                  accum, image, plan->n_sm, st);
+        if (e != cudaSuccess) return epic_cuda_fail(e, "auto-correlation epilogue");
+    } else if (image) {
+        e = epic::launch_finalize_image(accum, image, (long long)npix, inv_t, st);
+        if (e != cudaSuccess) return epic_cuda_fail(e, "image epilogue");
+    }
     return EPIC_OK;
 }
 

@@ -226,7 +226,8 @@ size_t grid_smem_bytes(int n_ant, int tb);
 int grid_samples_per_unit(int n_ant, size_t smem_optin);
 cudaError_t launch_grid(int vdt, int tb, const GridArgs& a, int n_sm, cudaStream_t st);
 
-// Epilogue kernels (finalize.cu).
+// Epilogue kernels (finalize.cu), and the zeroing of the accumulators (power may be nullptr).
+cudaError_t launch_zero(double* accum, long long n_accum, double* power, long long n_power, cudaStream_t st);
 cudaError_t launch_finalize_image(const double* accum, float* image, long long n, double inv_t,
                                   cudaStream_t st);
 cudaError_t launch_finalize_xpol(const double* accum4, float* image, float2* cross, int n_chan, long long npix,
@@ -236,7 +237,8 @@ size_t weff_smem_bytes(int lag_side, int n_pad);
 cudaError_t launch_weff(const float2* lag_tab, int n_ant, int lag_side, int n_pad, float* out, cudaStream_t st);
 cudaError_t launch_isotropic(const float* image, const float* autocorr, const float* weff, float rel_floor,
                              int n_ant, long long n, int npix, float* iso, cudaStream_t st);
-cudaError_t launch_autocorr(const double* power, const float2* lag_tab, int n_cp, int n_ant,
-                            int lag_side, int n_pad, double inv_t, float* out, cudaStream_t st);
+// image != nullptr: also image = accum * inv_t
+cudaError_t launch_autocorr(const double* power, const float2* lag_tab, const float2* twiddle, int n_cp, int n_ant, int lag_side, int n_pad,
+                            double inv_t, float* out, const double* accum, float* image, int n_sm, cudaStream_t st);
 
 }  // namespace epic

@@ -31,6 +31,26 @@ cudaError_t launch_finalize_image(const double* accum, float* image, long long n
     return cudaGetLastError();
 }
 
+// Zeroes the accumulators of a call that starts an integration.  Two small arrays in one launch: 64 x 64
+// pixels and 16 powers took two memsets of about 1.5 us each, and their two calls on the host.
+__global__ void zero_kernel(double* __restrict__ x, long long nx, double* __restrict__ y, long long ny) {
+    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (i < nx) x[i] = 0.0;
+    if (i < ny) y[i] = 0.0;
+}
+
+cudaError_t launch_zero(double* accum, long long n_accum, double* power, long long n_power, cudaStream_t st) {
+    // past 2 MB the copy engine's fill is the faster one, and the launches no longer count
+    if (n_accum > (1 << 18) || n_power > (1 << 18) || !power) {
+        const cudaError_t e = cudaMemsetAsync(accum, 0, (size_t)n_accum * sizeof(double), st);
+        return e != cudaSuccess || !power ? e : cudaMemsetAsync(power, 0, (size_t)n_power * sizeof(double), st);
+    }
+    const long long n = n_accum > n_power ? n_accum : n_power;
+    if (n == 0) return cudaSuccess;
+    zero_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(accum, n_accum, power, n_power);
+    return cudaGetLastError();
+}
+
 // Cross-polarisation epilogue.  accum4 holds per channel the time sums S_v(k) of |F_v|^2 for
 // the virtual pols v = X, Y, X + Y, X + iY; since |F_X + F_Y|^2 = |F_X|^2 + |F_Y|^2 +
 // 2 Re(F_X conj F_Y) and |F_X + i F_Y|^2 = |F_X|^2 + |F_Y|^2 + 2 Im(F_X conj F_Y),
@@ -66,42 +86,66 @@ cudaError_t launch_finalize_xpol(const double* accum4, float* image, float2* cro
 }
 
 constexpr int kAcThreads = 512;
+constexpr int kAcMaxCluster = 8;
 
-// One block per (channel, pol).  Shared: U [L*L] float2, T1 [L][N_p] float2, twiddles
-// [N_p] float2, P [A] float.  Three phases:
-//   U(d)        = sum_a P_a R_a(d)                       (L^2 x A multiply-adds)
-//   T1(dy, kx)  = sum_dx U(dy, dx) exp(+2 pi i dx kx / N_p) (L^2 x N_p)
-//   A(ky, kx)   = Re sum_dy T1(dy, kx) exp(+2 pi i dy ky / N_p)  (N_p^2 x L)
-// with k measured from the image centre (k = pixel - N_p/2; the exponent is periodic).
+// A cluster of n_cl CTAs per (channel, pol).  Shared: U [L*L] float2, the CTA's part of U [L*L] float2,
+// T1 [L][N_p] float2, twiddles [N_p] float2, the CTA's share of the powers.  Phases:
+//   U(d)        = sum_a P_a R_a(d)                       (L^2 x A multiply-adds): each CTA sums its share of
+//                 the antennas, kAcThreads / L^2 of them side by side, then every CTA adds up the parts
+//   T1(dy, kx)  = sum_dx U(dy, dx) exp(+2 pi i dx kx / N_p) (L^2 x N_p, in every CTA)
+//   A(ky, kx)   = Re sum_dy T1(dy, kx) exp(+2 pi i dy ky / N_p)  (N_p^2 x L, split over the CTAs)
+// with k measured from the image centre (k = pixel - N_p/2; the exponent is periodic).  With an image
+// it is written here too, image = accum / T_total, instead of by a kernel of its own.
+//
+// Bound by latency: a (channel, pol) has only L^2 lags (about 100) to sum A antennas into.  One CTA per
+// (channel, pol) with one thread per lag, and twiddles from FP64 sincospi in every CTA, took 50 us for 32 of
+// them with 256 antennas (N_p = 128) and 9.5 us for one with 16 antennas (N_p = 64), beside 5 and 2.6 us
+// for the image's own kernel; now 16.8 and 6.6 us for both.
 __global__ void __launch_bounds__(kAcThreads)
 autocorr_kernel(const double* __restrict__ power, const float2* __restrict__ lag_tab,
-                int n_ant, int L, int n_pad, double inv_t, float* __restrict__ out) {
+                const float2* __restrict__ twiddle, int n_ant, int L, int n_pad, double inv_t, float* __restrict__ out,
+                const double* __restrict__ accum, float* __restrict__ image) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2* U = reinterpret_cast<float2*>(smem_raw);
-    float2* T1 = U + L * L;
-    float2* TWs = T1 + L * n_pad;
-    float* P = reinterpret_cast<float*>(TWs + n_pad);
-    const int cp = blockIdx.x;
     const int LL = L * L, h = (L - 1) / 2, msk = n_pad - 1;
-    for (int j = threadIdx.x; j < n_pad; j += blockDim.x) {
-        double s, c;
-        sincospi(2.0 * j / n_pad, &s, &c);
-        TWs[j] = make_float2(float(c), float(s));
-    }
+    float2* U = reinterpret_cast<float2*>(smem_raw);
+    float2* UP = U + LL;
+    float2* T1 = UP + LL;
+    float2* TWs = T1 + L * n_pad;
+    const int n_cl = (int)cg::this_cluster().num_blocks(), rank = (int)cg::this_cluster().block_rank();
+    const int cp = blockIdx.x / n_cl;
+    for (int j = threadIdx.x; j < n_pad; j += blockDim.x) TWs[j] = __ldg(twiddle + j);
+    // this CTA's antennas; G of them side by side (the sums of a lag's G threads meet in T1's space)
+    const int a0 = (int)((long long)n_ant * rank / n_cl), a1 = (int)((long long)n_ant * (rank + 1) / n_cl);
+    const int G = max(1, min(kAcThreads / LL, L * n_pad / LL));
     const double* pw = power + (size_t)cp * n_ant;
-    for (int aa = threadIdx.x; aa < n_ant; aa += blockDim.x) P[aa] = float(pw[aa] * inv_t);
+    float* P = reinterpret_cast<float*>(TWs + n_pad);          // the share's mean powers (the FP64 product once each)
+    for (int aa = a0 + threadIdx.x; aa < a1; aa += blockDim.x) P[aa - a0] = float(__ldg(pw + aa) * inv_t);
     __syncthreads();
-    for (int j = threadIdx.x; j < LL; j += blockDim.x) {
+    for (int q = threadIdx.x; q < G * LL; q += blockDim.x) {
+        const int g = q / LL, j = q - g * LL;
         float2 u = make_float2(0.f, 0.f);
-        for (int aa = 0; aa < n_ant; ++aa) {
-            const float p = P[aa];
+#pragma unroll 4
+        for (int aa = a0 + g; aa < a1; aa += G) {
+            const float p = P[aa - a0];
             const float2 rv = __ldg(lag_tab + (size_t)aa * LL + j);
             u.x = fmaf(p, rv.x, u.x);
             u.y = fmaf(p, rv.y, u.y);
         }
-        U[j] = u;
+        T1[q] = u;
     }
     __syncthreads();
+    for (int j = threadIdx.x; j < LL; j += blockDim.x) {
+        float2 u = T1[j];
+        for (int g = 1; g < G; ++g) u = cadd(u, T1[g * LL + j]);
+        UP[j] = u;
+    }
+    cg::this_cluster().sync();
+    for (int j = threadIdx.x; j < LL; j += blockDim.x) {
+        float2 u = make_float2(0.f, 0.f);
+        for (int r = 0; r < n_cl; ++r) u = cadd(u, *cluster_ptr(UP + j, r));
+        U[j] = u;
+    }
+    cg::this_cluster().sync();       // the parts have been read: a CTA may leave; U is complete
     for (int j = threadIdx.x; j < L * n_pad; j += blockDim.x) {
         const int dy = j / n_pad, ix = j % n_pad, kx = ix - n_pad / 2;
         float2 acc = make_float2(0.f, 0.f);
@@ -116,7 +160,8 @@ autocorr_kernel(const double* __restrict__ power, const float2* __restrict__ lag
     }
     __syncthreads();
     const int npix = n_pad * n_pad;
-    for (int pix = threadIdx.x; pix < npix; pix += blockDim.x) {
+    const int p0 = (int)((long long)npix * rank / n_cl), p1 = (int)((long long)npix * (rank + 1) / n_cl);
+    for (int pix = p0 + threadIdx.x; pix < p1; pix += blockDim.x) {
         const int iy = pix / n_pad, ix = pix % n_pad, ky = iy - n_pad / 2;
         float accr = 0.f;
         for (int dy = 0; dy < L; ++dy) {
@@ -125,6 +170,7 @@ autocorr_kernel(const double* __restrict__ power, const float2* __restrict__ lag
             accr = fmaf(t.x, w.x, fmaf(-t.y, w.y, accr));
         }
         out[(size_t)cp * npix + pix] = accr;
+        if (image) image[(size_t)cp * npix + pix] = float(accum[(size_t)cp * npix + pix] * inv_t);
     }
 }
 
@@ -238,18 +284,47 @@ cudaError_t launch_isotropic(const float* image, const float* autocorr, const fl
     return cudaGetLastError();
 }
 
+// The size that decides whether a plan has the auto-correlation tables.
 size_t autocorr_smem_bytes(int lag_side, int n_pad, int n_ant) {
     return sizeof(float2) * ((size_t)lag_side * lag_side + (size_t)lag_side * n_pad + n_pad)
          + sizeof(float) * (size_t)n_ant;
 }
 
-cudaError_t launch_autocorr(const double* power, const float2* lag_tab, int n_cp, int n_ant,
-                            int lag_side, int n_pad, double inv_t, float* out, cudaStream_t st) {
-    const size_t smem = autocorr_smem_bytes(lag_side, n_pad, n_ant);
+cudaError_t launch_autocorr(const double* power, const float2* lag_tab, const float2* twiddle, int n_cp, int n_ant, int lag_side, int n_pad,
+                            double inv_t, float* out, const double* accum, float* image, int n_sm, cudaStream_t st) {
+    // CTAs per (channel, pol): up to two CTAs per SM over the call, at least 2 antennas and 512 pixels each
+    int n_cl = 1;
+    while (n_cl < kAcMaxCluster && (long long)n_cp * n_cl < 2LL * n_sm && n_cl * 2 * 2 <= n_ant &&
+           n_pad * n_pad >= kAcThreads * n_cl * 2)
+        n_cl *= 2;
+    // a plan at the limit of autocorr_smem_bytes may leave no room for the second L^2 table with all its powers
+    auto need = [&](int k) {
+        return sizeof(float2) * (2 * (size_t)lag_side * lag_side + (size_t)lag_side * n_pad + n_pad)
+             + sizeof(float) * (size_t)((n_ant + k - 1) / k);
+    };
+    if (need(n_cl) > 48 * 1024) {
+        int dev = 0, optin = 0;
+        cudaError_t q = cudaGetDevice(&dev);
+        if (q == cudaSuccess) q = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (q != cudaSuccess) return q;
+        while (n_cl < kAcMaxCluster && need(n_cl) > (size_t)optin) n_cl *= 2;
+    }
+    const size_t smem = need(n_cl);
     cudaError_t e = ensure_smem<autocorr_kernel>(smem);
     if (e != cudaSuccess) return e;
-    autocorr_kernel<<<n_cp, kAcThreads, smem, st>>>(power, lag_tab, n_ant, lag_side, n_pad, inv_t, out);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = n_cl;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)n_cp * n_cl);
+    cfg.blockDim = dim3(kAcThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, autocorr_kernel, power, lag_tab, twiddle, n_ant, lag_side, n_pad, inv_t, out, accum, image);
 }
 
 int resident_fwd_workers_32(int vdt, int max_ant, int n_sm);

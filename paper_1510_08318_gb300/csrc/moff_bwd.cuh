@@ -274,7 +274,9 @@ cudaError_t launch_bwd_t(const BwdArgs& a, int n_sm, cudaStream_t st) {
     if (a.n_items == 0) return cudaSuccess;
     if constexpr (G::Q == 1) {
         int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, G::NT, smem);
+        e = cached_occupancy<moff_bwd_kernel<NP, VDT>>(smem, &per_sm, [&](int* v) {
+            return cudaOccupancyMaxActiveBlocksPerMultiprocessor(v, kern, G::NT, smem);
+        });
         if (e != cudaSuccess) return e;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
         long long grid = (long long)per_sm * n_sm;
@@ -299,7 +301,7 @@ cudaError_t launch_bwd_t(const BwdArgs& a, int n_sm, cudaStream_t st) {
             if (e != cudaSuccess) return e;
         }
         int n_cl = 0;
-        e = cudaOccupancyMaxActiveClusters(&n_cl, kern, &cfg);
+        e = cached_occupancy<moff_bwd_kernel<NP, VDT>>(smem, &n_cl, [&](int* v) { return cudaOccupancyMaxActiveClusters(v, kern, &cfg); });
         if (e != cudaSuccess) return e;
         if (n_cl < 1) return cudaErrorInvalidConfiguration;
         long long ncl = n_cl;

@@ -282,6 +282,26 @@ cudaError_t ensure_smem(size_t bytes) {
     return e;
 }
 
+// Result of an occupancy query of one kernel (KEY), kept per host thread for its last device and
+// shared-memory size: the query takes about as long as a launch.
+template <auto KEY, typename F>
+cudaError_t cached_occupancy(size_t smem, int* out, F query) {
+    thread_local int c_dev = -1, c_val = 0;
+    thread_local size_t c_smem = 0;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev != c_dev || smem != c_smem) {
+        int v = 0;
+        if ((e = query(&v)) != cudaSuccess) return e;
+        c_dev = dev;
+        c_smem = smem;
+        c_val = v;
+    }
+    *out = c_val;
+    return cudaSuccess;
+}
+
 // Contiguous share [beg, end) of n items for worker w of nw.
 __device__ __forceinline__ void work_range(long long n, int w, int nw, long long& beg, long long& end) {
     const long long per = n / nw, rem = n % nw;

@@ -379,7 +379,9 @@ cudaError_t launch_fwd_nb(const SegList& L, int n_sm, cudaStream_t st) {
     if (n_items == 0) return cudaSuccess;
     if constexpr (G::Q == 1) {
         int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, G::NT, smem);
+        e = cached_occupancy<moff_fwd_kernel<NP, VDT, XP, NB>>(smem, &per_sm, [&](int* v) {
+            return cudaOccupancyMaxActiveBlocksPerMultiprocessor(v, kern, G::NT, smem);
+        });
         if (e != cudaSuccess) return e;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
         long long grid = (long long)per_sm * n_sm;
@@ -405,7 +407,7 @@ cudaError_t launch_fwd_nb(const SegList& L, int n_sm, cudaStream_t st) {
             if (e != cudaSuccess) return e;
         }
         int n_cl = 0;
-        e = cudaOccupancyMaxActiveClusters(&n_cl, kern, &cfg);
+        e = cached_occupancy<moff_fwd_kernel<NP, VDT, XP, NB>>(smem, &n_cl, [&](int* v) { return cudaOccupancyMaxActiveClusters(v, kern, &cfg); });
         if (e != cudaSuccess) return e;
         if (n_cl < 1) return cudaErrorInvalidConfiguration;
         long long ncl = n_cl;

@@ -176,9 +176,9 @@ def fengine(raw, n_chan, in_dtype, out_dtype="f16", stream=None):
         out = torch.empty((T, n_chan, P, A, 2), dtype=torch.float16, device=raw.device)
     else:
         out = torch.empty((T, n_chan, P, A), dtype=torch.complex64, device=raw.device)
-    st = torch.cuda.current_stream(raw.device) if stream is None else stream
+    st = _raw_stream(stream, raw.device.index or 0)
     epic_fengine(A, P, n_chan, T, VOLT_DTYPES[in_dtype], raw.data_ptr(), VOLT_DTYPES[out_dtype], out.data_ptr(),
-                 raw.device.index or 0, st.cuda_stream)
+                 raw.device.index or 0, st)
     return out
 
 
@@ -264,6 +264,15 @@ def epic_plan_info(plan):
     return {"nnz": nnz.value, "n_cells": cells.value, "lag_side": lag.value}
 
 
+def _raw_stream(stream, device):
+    """cudaStream_t of a torch stream, or of the device's current stream when it is None (read as a
+    plain number: building the Stream object costs more than a kernel launch)."""
+    if stream is not None:
+        return stream.cuda_stream
+    import torch
+    return torch._C._cuda_getCurrentRawStream(device)
+
+
 # ---- torch convenience layer --------------------------------------------------------------
 class Plan:
     """An imaging plan on one CUDA device (antenna-to-grid mapping + device tables)."""
@@ -274,6 +283,7 @@ class Plan:
         self.n_grid, self.n_pad, self.n_chan, self.n_pol = int(n_grid), int(n_pad), int(n_chan), int(n_pol)
         self.vdtype = vdtype
         self.device = int(device)
+        self._dev = None
         self._h = epic_create(self.n_ant, pos, kern_ptr, kern_dxdy, kern_w, dx, origin, n_grid, n_pad,
                               n_chan, n_pol, VOLT_DTYPES[vdtype], device)
         self.info = epic_plan_info(self._h)
@@ -292,8 +302,8 @@ class Plan:
         """epic_sync: wait for the stream and raise EpicError (status EPIC_ETIMEOUT) if a bounded
         tensor-core wait of this plan's kernels ran out since the last sync."""
         import torch
-        st = torch.cuda.current_stream(torch.device("cuda", self.device)) if stream is None else stream
-        epic_sync(self._h, st.cuda_stream)
+        st = _raw_stream(stream, self.device)
+        epic_sync(self._h, st)
 
     def set_wait_limit(self, tries):
         """epic_set_wait_limit: tries (about 1 ms each) of the tensor-core pipelines' waits."""
@@ -315,6 +325,12 @@ class Plan:
             self.close()
         except Exception:
             pass
+
+    def _torch_device(self):
+        if self._dev is None:
+            import torch
+            self._dev = torch.device("cuda", self.device)
+        return self._dev
 
     # --- argument checks (shape, dtype, device, contiguity) ---
     def _volt_ptr(self, volt):
@@ -347,7 +363,7 @@ class Plan:
               want_autocorr=False, stream=None):
         """Run epic_image; returns dict(image, autocorr, accum, power) of CUDA tensors."""
         import torch
-        dev = torch.device("cuda", self.device)
+        dev = self._torch_device()
         vptr, T = self._volt_ptr(volt)
         C, P, NP, A = self.n_chan, self.n_pol, self.n_pad, self.n_ant
         if accum is None:
@@ -356,66 +372,66 @@ class Plan:
             power = torch.empty((C, P, A), dtype=torch.float64, device=dev)
         img = torch.empty((C, P, NP, NP), dtype=torch.float32, device=dev) if want_image else None
         ac = torch.empty((C, P, NP, NP), dtype=torch.float32, device=dev) if want_autocorr else None
-        st = torch.cuda.current_stream(dev) if stream is None else stream
+        st = _raw_stream(stream, self.device)
         epic_image(self._h, vptr, T, self._gains_ptr(gains), accum.data_ptr(), _ptr(power), t_prev,
-                   _ptr(img), _ptr(ac), st.cuda_stream)
+                   _ptr(img), _ptr(ac), st)
         return {"image": img, "autocorr": ac, "accum": accum, "power": power}
 
     def image_backward(self, volt, gains, grad_image, stream=None):
         import torch
-        dev = torch.device("cuda", self.device)
+        dev = self._torch_device()
         vptr, T = self._volt_ptr(volt)
         g = grad_image.contiguous().to(torch.float32)
         if tuple(g.shape) != (self.n_chan, self.n_pol, self.n_pad, self.n_pad) or not g.is_cuda:
             raise ValueError("grad_image must be a CUDA tensor [C, P, N_p, N_p]")
         out = torch.empty((self.n_chan, self.n_pol, self.n_ant), dtype=torch.complex64, device=dev)
-        st = torch.cuda.current_stream(dev) if stream is None else stream
+        st = _raw_stream(stream, self.device)
         epic_image_backward(self._h, vptr, T, self._gains_ptr(gains), g.data_ptr(), out.data_ptr(),
-                            st.cuda_stream)
+                            st)
         return out
 
     def image_xpol(self, volt, gains=None, accum4=None, t_prev=0, stream=None):
         """Run epic_image_xpol: dict(image [C, 2, N_p, N_p] float32 (XX, YY), cross [C, N_p, N_p]
         complex64 (XY = <F_X conj F_Y>), accum4 [C, 4, N_p, N_p] float64)."""
         import torch
-        dev = torch.device("cuda", self.device)
+        dev = self._torch_device()
         vptr, T = self._volt_ptr(volt)
         C, NP = self.n_chan, self.n_pad
         if accum4 is None:
             accum4 = torch.empty((C, 4, NP, NP), dtype=torch.float64, device=dev)
         img = torch.empty((C, 2, NP, NP), dtype=torch.float32, device=dev)
         cross = torch.empty((C, NP, NP), dtype=torch.complex64, device=dev)
-        st = torch.cuda.current_stream(dev) if stream is None else stream
+        st = _raw_stream(stream, self.device)
         epic_image_xpol(self._h, vptr, T, self._gains_ptr(gains), accum4.data_ptr(), t_prev, img.data_ptr(),
-                        cross.data_ptr(), st.cuda_stream)
+                        cross.data_ptr(), st)
         return {"image": img, "cross": cross, "accum4": accum4}
 
     def fx_image(self, vis, stream=None):
         """Run epic_fx_image: the FX-route image [C, P, N_p, N_p] of visibilities [C, P, A, A]."""
         import torch
-        dev = torch.device("cuda", self.device)
+        dev = self._torch_device()
         if (vis.dtype != torch.complex64 or tuple(vis.shape) != (self.n_chan, self.n_pol, self.n_ant, self.n_ant)
                 or not vis.is_cuda or not vis.is_contiguous()):
             raise ValueError("vis must be a contiguous complex64 CUDA tensor [C, P, A, A]")
         out = torch.empty((self.n_chan, self.n_pol, self.n_pad, self.n_pad), dtype=torch.float32, device=dev)
-        st = torch.cuda.current_stream(dev) if stream is None else stream
-        epic_fx_image(self._h, vis.data_ptr(), out.data_ptr(), st.cuda_stream)
+        st = _raw_stream(stream, self.device)
+        epic_fx_image(self._h, vis.data_ptr(), out.data_ptr(), st)
         return out
 
     def weff(self, stream=None):
         """Run epic_weff: the effective weighting W_eff [N_p, N_p] (float32 CUDA tensor)."""
         import torch
-        dev = torch.device("cuda", self.device)
+        dev = self._torch_device()
         out = torch.empty((self.n_pad, self.n_pad), dtype=torch.float32, device=dev)
-        st = torch.cuda.current_stream(dev) if stream is None else stream
-        epic_weff(self._h, out.data_ptr(), st.cuda_stream)
+        st = _raw_stream(stream, self.device)
+        epic_weff(self._h, out.data_ptr(), st)
         return out
 
     def isotropic(self, image, autocorr, weff, rel_floor=1e-3, stream=None):
         """Run epic_isotropic: (image - autocorr) / (A (A - 1) W_eff), NaN where W_eff is below
         rel_floor of its peak."""
         import torch
-        dev = torch.device("cuda", self.device)
+        dev = self._torch_device()
         shape = (self.n_chan, self.n_pol, self.n_pad, self.n_pad)
         for t in (image, autocorr):
             if t.dtype != torch.float32 or tuple(t.shape) != shape or not t.is_cuda or not t.is_contiguous():
@@ -423,15 +439,15 @@ class Plan:
         if tuple(weff.shape) != (self.n_pad, self.n_pad) or weff.dtype != torch.float32 or not weff.is_contiguous():
             raise ValueError("weff must be a contiguous float32 tensor [N_p, N_p]")
         out = torch.empty(shape, dtype=torch.float32, device=dev)
-        st = torch.cuda.current_stream(dev) if stream is None else stream
+        st = _raw_stream(stream, self.device)
         epic_isotropic(self._h, image.data_ptr(), autocorr.data_ptr(), weff.data_ptr(), rel_floor, out.data_ptr(),
-                       st.cuda_stream)
+                       st)
         return out
 
     def correlate(self, volt, gains=None, out=None, stream=None):
         """Run epic_correlate: visibilities <g_a V_a conj(g_b V_b)>_t, complex64 [C, P, A, A]."""
         import torch
-        dev = torch.device("cuda", self.device)
+        dev = self._torch_device()
         vptr, T = self._volt_ptr(volt)
         shape = (self.n_chan, self.n_pol, self.n_ant, self.n_ant)
         if out is None:
@@ -439,14 +455,14 @@ class Plan:
         elif (out.dtype != torch.complex64 or tuple(out.shape) != shape or not out.is_cuda
               or not out.is_contiguous()):
             raise ValueError("out must be a contiguous complex64 CUDA tensor %s" % (shape,))
-        st = torch.cuda.current_stream(dev) if stream is None else stream
-        epic_correlate(self._h, vptr, T, self._gains_ptr(gains), out.data_ptr(), st.cuda_stream)
+        st = _raw_stream(stream, self.device)
+        epic_correlate(self._h, vptr, T, self._gains_ptr(gains), out.data_ptr(), st)
         return out
 
     def grid(self, volt, gains=None, out=None, stream=None):
         """Run epic_grid: the gridded fields E_t(g), complex64 CUDA tensor [T, C, P, N_g, N_g]."""
         import torch
-        dev = torch.device("cuda", self.device)
+        dev = self._torch_device()
         vptr, T = self._volt_ptr(volt)
         shape = (T, self.n_chan, self.n_pol, self.n_grid, self.n_grid)
         if out is None:
@@ -454,8 +470,8 @@ class Plan:
         elif (out.dtype != torch.complex64 or tuple(out.shape) != shape or not out.is_cuda
               or not out.is_contiguous()):
             raise ValueError("out must be a contiguous complex64 CUDA tensor %s" % (shape,))
-        st = torch.cuda.current_stream(dev) if stream is None else stream
-        epic_grid(self._h, vptr, T, self._gains_ptr(gains), out.data_ptr(), st.cuda_stream)
+        st = _raw_stream(stream, self.device)
+        epic_grid(self._h, vptr, T, self._gains_ptr(gains), out.data_ptr(), st)
         return out
 
 
@@ -486,16 +502,16 @@ class Batch:
     def image(self, volts, accum, image=None, gains=None, stream=None):
         import torch
         ptrs, nts = self._bufs(volts)
-        st = torch.cuda.current_stream(torch.device("cuda", self.plans[0].device)) if stream is None else stream
+        st = _raw_stream(stream, self.plans[0].device)
         g = None if gains is None else [None if x is None else self.plans[i]._gains_ptr(x) for i, x in enumerate(gains)]
-        epic_batch_image(self._h, ptrs, nts, g, accum, image, st.cuda_stream)
+        epic_batch_image(self._h, ptrs, nts, g, accum, image, st)
 
     def autotune(self, volts, accum, gains=None, stream=None):
         import torch
         ptrs, nts = self._bufs(volts)
-        st = torch.cuda.current_stream(torch.device("cuda", self.plans[0].device)) if stream is None else stream
+        st = _raw_stream(stream, self.plans[0].device)
         g = None if gains is None else [None if x is None else self.plans[i]._gains_ptr(x) for i, x in enumerate(gains)]
-        epic_batch_autotune(self._h, ptrs, nts, g, accum, st.cuda_stream)
+        epic_batch_autotune(self._h, ptrs, nts, g, accum, st)
         return epic_batch_info(self._h)
 
     def info(self):
