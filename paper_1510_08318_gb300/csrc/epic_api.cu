@@ -60,6 +60,14 @@ void free_plan(epic_plan* p) {
     cudaFree(p->wbase);
     cudaFree(p->went);
     cudaFree(p->wwim);
+    cudaFree(p->hg_run);
+    cudaFree(p->hg_w);
+    cudaFree(p->hg_wim);
+    cudaFree(p->hg_key);
+    cudaFree(p->hg_empty);
+    cudaFree(p->hg_ant_ptr);
+    cudaFree(p->hg_ant_ent);
+    cudaFree(p->hg_ant_wim);
     cudaFree(p->ant_ptr);
     cudaFree(p->ant_ent);
     cudaFree(p->ant_wim);
@@ -151,6 +159,7 @@ epic::FwdArgs epic_plan_fwd_args(const epic_plan* plan, const void* volt, int n_
     a.wsum_max = plan->wsum_max;
     a.status = plan->status;
     a.wait_tries = plan->wait_tries;
+    a.half = plan->half_gather();
     return a;
 }
 
@@ -346,32 +355,53 @@ epic_status epic_create(epic_plan** plan, int n_ant, const double* pos_xy, const
             dwpk[q] = ((uint32_t)__half_as_ushort(__float2half_rn(dwre[q])) << 16) | (uint32_t)dant[q];
     }
 
+    // gridding table of the half-image kernels
+    int smem_half = 0;
+    cudaDeviceGetAttribute(&smem_half, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+    p->half256 = n_pad == 256 && epic::half256_fits(n_ant, (size_t)smem_half);
+    std::vector<int4> hrun;
+    std::vector<float2> hw, hwim;
+    std::vector<uint32_t> hkey;
+    std::vector<uint16_t> hempty;
+    if (p->half256) epic::half256_tables(cptr, cent, cwim, hrun, hw, hwim, hkey, hempty);
+
     // antenna-major CSR per row block (degridding side of the adjoint); cells are stored as
     // offsets into the adjoint kernel's shared-memory row buffer
-    const int rows = epic::grid_rows_per_block(n_pad);
-    const int nq = NG / rows;
-    const int rxs = epic::exchange_row_stride(n_pad);
-    std::vector<std::vector<std::pair<int2, float>>> per_ant((size_t)nq * n_ant);
-    for (const MapEntry& e : m) {
-        const int gy = e.cell / NG, gx = e.cell % NG;
-        const int q = gy / rows;
-        per_ant[(size_t)q * n_ant + e.ant].push_back({pack_entry(e.w, (gy - q * rows) * rxs + gx), float(e.w.imag())});
-    }
-    std::vector<int> aptr((size_t)nq * (n_ant + 1), 0);
-    std::vector<int2> aent;
     std::vector<float> awim;
-    aent.reserve(m.size());
-    awim.reserve(m.size());
-    for (int q = 0; q < nq; ++q) {
-        aptr[(size_t)q * (n_ant + 1)] = (int)aent.size();
-        for (int a = 0; a < n_ant; ++a) {
-            for (auto& pe : per_ant[(size_t)q * n_ant + a]) {
-                aent.push_back(pe.first);
-                awim.push_back(pe.second);
-            }
-            aptr[(size_t)q * (n_ant + 1) + a + 1] = (int)aent.size();
+    auto antenna_major = [&](int rows, int stride, std::vector<int>& aptr, std::vector<int2>& aent) {
+        const int nq = NG / rows;
+        std::vector<std::vector<std::pair<int2, float>>> per_ant((size_t)nq * n_ant);
+        for (const MapEntry& e : m) {
+            const int gy = e.cell / NG, gx = e.cell % NG;
+            const int q = gy / rows;
+            per_ant[(size_t)q * n_ant + e.ant].push_back({pack_entry(e.w, (gy - q * rows) * stride + gx), float(e.w.imag())});
         }
+        aptr.assign((size_t)nq * (n_ant + 1), 0);
+        aent.reserve(m.size());
+        awim.clear();
+        awim.reserve(m.size());
+        for (int q = 0; q < nq; ++q) {
+            aptr[(size_t)q * (n_ant + 1)] = (int)aent.size();
+            for (int a = 0; a < n_ant; ++a) {
+                for (auto& pe : per_ant[(size_t)q * n_ant + a]) {
+                    aent.push_back(pe.first);
+                    awim.push_back(pe.second);
+                }
+                aptr[(size_t)q * (n_ant + 1) + a + 1] = (int)aent.size();
+            }
+        }
+    };
+    // the half-image kernels hold the whole grid: one block, its own row stride
+    std::vector<int> haptr;
+    std::vector<int2> haent;
+    std::vector<float> hawim;
+    if (p->half256) {
+        antenna_major(NG, epic::half256_row_stride(), haptr, haent);
+        hawim = awim;
     }
+    std::vector<int> aptr;
+    std::vector<int2> aent;
+    antenna_major(epic::grid_rows_per_block(n_pad), epic::exchange_row_stride(n_pad), aptr, aent);
 
     // per-antenna footprint auto-correlation R_a(d) on the L x L lag window
     std::vector<std::vector<const MapEntry*>> by_ant(n_ant);
@@ -458,6 +488,11 @@ epic_status epic_create(epic_plan** plan, int n_ant, const double* pos_xy, const
         (SL > 0 && ((e = upload(&p->wlane, wlane)) != cudaSuccess || (e = upload(&p->wbase, wbase)) != cudaSuccess ||
                     (e = upload(&p->went, went)) != cudaSuccess ||
                     (complex_w && (e = upload(&p->wwim, wwim)) != cudaSuccess))) ||
+        (p->half256 && ((e = upload(&p->hg_run, hrun)) != cudaSuccess || (e = upload(&p->hg_w, hw)) != cudaSuccess ||
+                        (e = upload(&p->hg_key, hkey)) != cudaSuccess || (e = upload(&p->hg_empty, hempty)) != cudaSuccess ||
+                        (e = upload(&p->hg_ant_ptr, haptr)) != cudaSuccess || (e = upload(&p->hg_ant_ent, haent)) != cudaSuccess ||
+                        (complex_w && ((e = upload(&p->hg_wim, hwim)) != cudaSuccess ||
+                                       (e = upload(&p->hg_ant_wim, hawim)) != cudaSuccess)))) ||
         (dp_ok && ((e = upload(&p->dp_lane, plane)) != cudaSuccess || (e = upload(&p->dp_slot, pslot)) != cudaSuccess ||
                    (e = upload(&p->dp_w, pw)) != cudaSuccess || (e = upload(&p->dp_ant, pant)) != cudaSuccess ||
                    (complex_w && (e = upload(&p->dp_wim, pwim)) != cudaSuccess))) ||
@@ -826,6 +861,7 @@ epic_status epic_image_backward(const epic_plan* plan, const void* volt, int n_t
     a.grad_gains = reinterpret_cast<float2*>(grad_gains);
     a.n_items = (long long)cp * n_time;
     a.scale = float(2.0 / double(n_time));
+    a.half = plan->half_gather();
     return launch_bwd(plan, a, st);
 }
 

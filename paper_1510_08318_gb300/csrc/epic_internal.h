@@ -6,6 +6,21 @@
 
 namespace epic {
 
+// Gridding table of the half-image kernels (N_p = 256, moff_half256.cu): 256 slots of 32 cell pairs (x, y),
+// (x, y + 1), y even, walked by 16 warps; an entry is an antenna with its weights on both cells.
+struct HalfGather {
+    const int4* run = nullptr;      // [16] {first entry, steps of 32 entries, first empty place, slots of empty
+                                    // places} of each warp
+    const float2* w = nullptr;      // weights on (x, y) and (x, y + 1), real parts
+    const float2* wim = nullptr;    // imaginary parts, or nullptr
+    const uint32_t* key = nullptr;  // antenna, and at a pair's last step its place in shared memory
+    const uint16_t* empty = nullptr;   // places of the pairs that no antenna reaches
+    // antenna-major CSR of the adjoint's degridding, as in BwdArgs, over the whole grid
+    const int* ant_ptr = nullptr;
+    const int2* ant_ent = nullptr;
+    const float* ant_wim = nullptr;
+};
+
 // Everything a launch needs, all device pointers.
 struct FwdArgs {
     const void* volt;          // [T][C][P][A] raw voltages
@@ -31,6 +46,7 @@ struct FwdArgs {
     int* status;               // device status word of the plan (kernels with bounded waits OR in
                                // kStatus* bits when a wait runs out), or nullptr
     int wait_tries;            // tries of each bounded wait of the pipeline (about 1 ms each)
+    HalfGather half;           // N_p = 256, antennas that fit the half-image kernels
 };
 
 // Bits of a plan's device status word, set by a kernel whose bounded wait ran out (the call's
@@ -77,6 +93,7 @@ struct BwdArgs {
     float2* grad_gains;        // [CP][A]
     long long n_items;
     float scale;               // 2 / T
+    HalfGather half;           // N_p = 256: set when the half-image kernels are used
 };
 
 // F-engine (fengine.cu): per-antenna temporal DFT of blocks of C samples.
@@ -142,6 +159,16 @@ cudaError_t launch_bwd_64(int vdt, const BwdArgs& a, int n_sm, cudaStream_t st);
 cudaError_t launch_bwd_128(int vdt, const BwdArgs& a, int n_sm, cudaStream_t st);
 cudaError_t launch_bwd_256(int vdt, const BwdArgs& a, int n_sm, cudaStream_t st);
 cudaError_t launch_bwd_512(int vdt, const BwdArgs& a, int n_sm, cudaStream_t st);
+
+// Half-image form at N_p = 256 (moff_half256.cu); fits: whether the antennas fit its shared memory (both
+// kernels); row stride (float2) of the grid its degridding reads.
+bool half256_fits(int n_ant, size_t smem_optin);
+void half256_tables(const std::vector<int>& cptr, const std::vector<int2>& cent, const std::vector<float>& cwim,
+                    std::vector<int4>& run, std::vector<float2>& w, std::vector<float2>& wim,
+                    std::vector<uint32_t>& key, std::vector<uint16_t>& empty);
+int half256_row_stride();
+cudaError_t launch_half256_fwd(int vdt, const SegList& L, int n_sm, cudaStream_t st);
+cudaError_t launch_half256_bwd(int vdt, const BwdArgs& a, int n_sm, cudaStream_t st);
 
 // CTAs (Q = 1) or clusters (Q > 1) of the forward kernel resident on the whole GPU.
 int resident_fwd_workers(int n_pad, int vdt, int max_ant, int n_sm);

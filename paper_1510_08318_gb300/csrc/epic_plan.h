@@ -34,6 +34,18 @@ struct epic_plan {
     mutable float2* fx_vis_t = nullptr;
     mutable float2* fx_u = nullptr;
     mutable int64_t fx_lag_n = -1;   // entries; -1 until built
+    bool half256 = false;        // N_p = 256 and the antennas fit the half-image kernels
+    int4* hg_run = nullptr;      // their gridding table (epic::HalfGather)
+    float2* hg_w = nullptr;
+    float2* hg_wim = nullptr;
+    uint32_t* hg_key = nullptr;
+    uint16_t* hg_empty = nullptr;
+    int* hg_ant_ptr = nullptr;
+    int2* hg_ant_ent = nullptr;
+    float* hg_ant_wim = nullptr;
+    epic::HalfGather half_gather() const {
+        return epic::HalfGather{hg_run, hg_w, hg_wim, hg_key, hg_empty, hg_ant_ptr, hg_ant_ent, hg_ant_wim};
+    }
     int* ant_ptr = nullptr;
     int2* ant_ent = nullptr;
     float* ant_wim = nullptr;
