@@ -355,7 +355,7 @@ epic_status epic_create(epic_plan** plan, int n_ant, const double* pos_xy, const
             dwpk[q] = ((uint32_t)__half_as_ushort(__float2half_rn(dwre[q])) << 16) | (uint32_t)dant[q];
     }
 
-    // gridding table of the half-image kernels
+    // gridding runs of the kernels that walk cell pairs
     int smem_half = 0;
     cudaDeviceGetAttribute(&smem_half, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
     p->half256 = n_pad == 256 && epic::half256_fits(n_ant, (size_t)smem_half);
@@ -363,7 +363,9 @@ epic_status epic_create(epic_plan** plan, int n_ant, const double* pos_xy, const
     std::vector<float2> hw, hwim;
     std::vector<uint32_t> hkey;
     std::vector<uint16_t> hempty;
+    p->rows512 = n_pad == 512 && epic::twopass_rows2_fits(n_ant, (size_t)smem_half);
     if (p->half256) epic::half256_tables(cptr, cent, cwim, hrun, hw, hwim, hkey, hempty);
+    if (p->rows512) epic::twopass_tables(cptr, cent, cwim, hrun, hw, hwim, hkey, hempty);
 
     // antenna-major CSR per row block (degridding side of the adjoint); cells are stored as
     // offsets into the adjoint kernel's shared-memory row buffer
@@ -488,11 +490,12 @@ epic_status epic_create(epic_plan** plan, int n_ant, const double* pos_xy, const
         (SL > 0 && ((e = upload(&p->wlane, wlane)) != cudaSuccess || (e = upload(&p->wbase, wbase)) != cudaSuccess ||
                     (e = upload(&p->went, went)) != cudaSuccess ||
                     (complex_w && (e = upload(&p->wwim, wwim)) != cudaSuccess))) ||
-        (p->half256 && ((e = upload(&p->hg_run, hrun)) != cudaSuccess || (e = upload(&p->hg_w, hw)) != cudaSuccess ||
-                        (e = upload(&p->hg_key, hkey)) != cudaSuccess || (e = upload(&p->hg_empty, hempty)) != cudaSuccess ||
-                        (e = upload(&p->hg_ant_ptr, haptr)) != cudaSuccess || (e = upload(&p->hg_ant_ent, haent)) != cudaSuccess ||
-                        (complex_w && ((e = upload(&p->hg_wim, hwim)) != cudaSuccess ||
-                                       (e = upload(&p->hg_ant_wim, hawim)) != cudaSuccess)))) ||
+        ((p->half256 || p->rows512) &&
+         ((e = upload(&p->hg_run, hrun)) != cudaSuccess || (e = upload(&p->hg_w, hw)) != cudaSuccess ||
+          (e = upload(&p->hg_key, hkey)) != cudaSuccess || (e = upload(&p->hg_empty, hempty)) != cudaSuccess ||
+          (complex_w && (e = upload(&p->hg_wim, hwim)) != cudaSuccess))) ||
+        (p->half256 && ((e = upload(&p->hg_ant_ptr, haptr)) != cudaSuccess || (e = upload(&p->hg_ant_ent, haent)) != cudaSuccess ||
+                        (complex_w && (e = upload(&p->hg_ant_wim, hawim)) != cudaSuccess))) ||
         (dp_ok && ((e = upload(&p->dp_lane, plane)) != cudaSuccess || (e = upload(&p->dp_slot, pslot)) != cudaSuccess ||
                    (e = upload(&p->dp_w, pw)) != cudaSuccess || (e = upload(&p->dp_ant, pant)) != cudaSuccess ||
                    (complex_w && (e = upload(&p->dp_wim, pwim)) != cudaSuccess))) ||

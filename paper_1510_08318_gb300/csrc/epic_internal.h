@@ -6,11 +6,14 @@
 
 namespace epic {
 
-// Gridding table of the half-image kernels (N_p = 256, moff_half256.cu): 256 slots of 32 cell pairs (x, y),
-// (x, y + 1), y even, walked by 16 warps; an entry is an antenna with its weights on both cells.
+// Gridding runs of the kernels that walk cell pairs (x, y), (x, y + 1), y even: the half-image kernels at
+// N_p = 256 (one round of all 128 rows, 16 warps) and the two-pass form at N_p = 512 (16 rounds of 16 rows, 8
+// warps each); an entry is an antenna with its weights on both cells.
+constexpr int kGridAhead = 8;                    // entries of a run are read this many steps ahead
+constexpr uint32_t kGridLast = 0x80000000u;      // key: antenna | place << 16 | kGridLast at a pair's last step
 struct HalfGather {
-    const int4* run = nullptr;      // [16] {first entry, steps of 32 entries, first empty place, slots of empty
-                                    // places} of each warp
+    const int4* run = nullptr;      // [rounds][warps] {first entry, steps of 32 entries (a multiple of kGridAhead),
+                                    // first empty place, slots of empty places} of each warp
     const float2* w = nullptr;      // weights on (x, y) and (x, y + 1), real parts
     const float2* wim = nullptr;    // imaginary parts, or nullptr
     const uint32_t* key = nullptr;  // antenna, and at a pair's last step its place in shared memory
@@ -46,7 +49,7 @@ struct FwdArgs {
     int* status;               // device status word of the plan (kernels with bounded waits OR in
                                // kStatus* bits when a wait runs out), or nullptr
     int wait_tries;            // tries of each bounded wait of the pipeline (about 1 ms each)
-    HalfGather half;           // N_p = 256, antennas that fit the half-image kernels
+    HalfGather half;           // N_p = 256 and 512, antennas that fit the kernels that walk cell pairs
 };
 
 // Bits of a plan's device status word, set by a kernel whose bounded wait ran out (the call's
@@ -163,6 +166,9 @@ cudaError_t launch_bwd_512(int vdt, const BwdArgs& a, int n_sm, cudaStream_t st)
 // Half-image form at N_p = 256 (moff_half256.cu); fits: whether the antennas fit its shared memory (both
 // kernels); row stride (float2) of the grid its degridding reads.
 bool half256_fits(int n_ant, size_t smem_optin);
+void pair_run_tables(int ng, int rows, int stride, int warps, int per, const std::vector<int>& cptr, const std::vector<int2>& cent,
+                     const std::vector<float>& cwim, std::vector<int4>& run, std::vector<float2>& w,
+                     std::vector<float2>& wim, std::vector<uint32_t>& key, std::vector<uint16_t>& empty);
 void half256_tables(const std::vector<int>& cptr, const std::vector<int2>& cent, const std::vector<float>& cwim,
                     std::vector<int4>& run, std::vector<float2>& w, std::vector<float2>& wim,
                     std::vector<uint32_t>& key, std::vector<uint16_t>& empty);
@@ -245,6 +251,11 @@ cudaError_t launch_dftgemm256(int vdt, const FwdArgs& a, const void* wtab, const
 // items in chunks of chunk_items, scratch of twopass_scratch_bytes(chunk_items), caller-owned.
 size_t twopass_scratch_bytes(int chunk_items);
 size_t twopass_rows_smem_bytes(int max_ant);
+// the two-sample row pass: whether the antennas fit it, and its gridding runs
+bool twopass_rows2_fits(int n_ant, size_t smem_optin);
+void twopass_tables(const std::vector<int>& cptr, const std::vector<int2>& cent, const std::vector<float>& cwim,
+                    std::vector<int4>& run, std::vector<float2>& w, std::vector<float2>& wim,
+                    std::vector<uint32_t>& key, std::vector<uint16_t>& empty);
 cudaError_t launch_fwd512_twopass(int vdt, const SegList& L, int n_sm, cudaStream_t st, float2* scratch,
                                   int chunk_items);
 

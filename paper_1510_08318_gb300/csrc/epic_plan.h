@@ -35,7 +35,8 @@ struct epic_plan {
     mutable float2* fx_u = nullptr;
     mutable int64_t fx_lag_n = -1;   // entries; -1 until built
     bool half256 = false;        // N_p = 256 and the antennas fit the half-image kernels
-    int4* hg_run = nullptr;      // their gridding table (epic::HalfGather)
+    bool rows512 = false;        // N_p = 512 and the antennas fit the two-sample row pass
+    int4* hg_run = nullptr;      // gridding runs of either (epic::HalfGather)
     float2* hg_w = nullptr;
     float2* hg_wim = nullptr;
     uint32_t* hg_key = nullptr;

@@ -50,7 +50,6 @@ constexpr int ROWF2 = 2 * RBS;         // row stride in float2
 
 constexpr size_t kRB = (size_t)NG * RBS * 16, kRX = (size_t)NPAIR * RXS * 8;
 constexpr size_t kTables = 2 * 128 * sizeof(float2);
-constexpr int NSLOT = 256;             // gridding slots of 32 cell pairs
 constexpr size_t kFixed = kRB + kRX + kTables + 16;
 constexpr size_t fwd_smem(int n_ant) { return kFixed + (size_t)n_ant * (sizeof(float2) + sizeof(float)); }
 constexpr size_t bwd_smem(int n_ant) { return kFixed + (size_t)n_ant * 2 * sizeof(float2); }
@@ -108,23 +107,21 @@ __device__ __forceinline__ P2 mul_wc(const P2& x, float2 w) {
 // RB[68 y + x].  A lane takes the cell pairs (x, y), (x, y + 1) of its warp's slots one after the other: each step is
 // 32 entries, an antenna with its weights on both cells and, at a pair's last step, the pair's place in RB.  The
 // table does not fit beside the transform's buffers and comes from L2 in every unit: the warp's steps are one run
-// of it, read kAhead steps ahead, in 12 bytes an entry (16 bytes an entry, with the cells that no antenna reaches
+// of it, read kGridAhead steps ahead, in 12 bytes an entry (16 bytes an entry, with the cells that no antenna reaches
 // among them, took the kernel's L2 reads to 6 TB/s and a third of its time).
-constexpr int kAhead = 8;
-constexpr uint32_t kLast = 0x80000000u;      // key: antenna | place << 16 | kLast at a pair's last step
 template <bool CW>
 __device__ __forceinline__ void grid_pairs(const Smem& m, const HalfGather& g, int tid, const float2* VB) {
     const int lane = tid & 31, warp = tid >> 5;
-    const int4 run = __ldg(g.run + warp);                  // first entry, steps (a multiple of kAhead), first empty
+    const int4 run = __ldg(g.run + warp);                  // first entry, steps (a multiple of kGridAhead), first empty
                                                            // place, slots of empty places
     const float2* wt = g.w + run.x + lane;
     const float2* wim = CW ? g.wim + run.x + lane : nullptr;
     const uint32_t* key = g.key + run.x + lane;
-    float2 w[kAhead], wi[CW ? kAhead : 1];
-    uint32_t ky[kAhead];
+    float2 w[kGridAhead], wi[CW ? kGridAhead : 1];
+    uint32_t ky[kGridAhead];
     auto load = [&](int k) {
 #pragma unroll
-        for (int u = 0; u < kAhead; ++u) {
+        for (int u = 0; u < kGridAhead; ++u) {
             w[u] = __ldg(wt + 32 * (k + u));
             ky[u] = __ldg(key + 32 * (k + u));
             if constexpr (CW) wi[u] = __ldg(wim + 32 * (k + u));
@@ -134,18 +131,18 @@ __device__ __forceinline__ void grid_pairs(const Smem& m, const HalfGather& g, i
     for (int z = 0; z < run.w; ++z) m.RB[__ldg(g.empty + run.z + 32 * z + lane)] = make_float4(0.f, 0.f, 0.f, 0.f);
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
-    for (int k = 0; k < run.y; k += kAhead) {
-        float2 cw[kAhead], ci[CW ? kAhead : 1];
-        uint32_t ck[kAhead];
+    for (int k = 0; k < run.y; k += kGridAhead) {
+        float2 cw[kGridAhead], ci[CW ? kGridAhead : 1];
+        uint32_t ck[kGridAhead];
 #pragma unroll
-        for (int u = 0; u < kAhead; ++u) {
+        for (int u = 0; u < kGridAhead; ++u) {
             cw[u] = w[u];
             ck[u] = ky[u];
             if constexpr (CW) ci[u] = wi[u];
         }
-        if (k + kAhead < run.y) load(k + kAhead);
+        if (k + kGridAhead < run.y) load(k + kGridAhead);
 #pragma unroll
-        for (int u = 0; u < kAhead; ++u) {
+        for (int u = 0; u < kGridAhead; ++u) {
             const float2 v = VB[ck[u] & 0xffffu];
             s.x = fmaf(cw[u].x, v.x, s.x);
             s.y = fmaf(cw[u].y, v.x, s.y);
@@ -157,7 +154,7 @@ __device__ __forceinline__ void grid_pairs(const Smem& m, const HalfGather& g, i
                 s.z = fmaf(ci[u].x, v.x, s.z);
                 s.w = fmaf(ci[u].y, v.x, s.w);
             }
-            if (ck[u] & kLast) {                           // the same for all lanes
+            if (ck[u] & kGridLast) {                           // the same for all lanes
                 m.RB[(ck[u] >> 16) & 0x7fffu] = s;
                 s = make_float4(0.f, 0.f, 0.f, 0.f);
             }
@@ -667,103 +664,113 @@ cudaError_t launch_bwd(const BwdArgs& a, int n_sm, cudaStream_t st) {
 
 }  // namespace half256
 
-// Slots of the gridding: the 16-byte word of (x, y), y even, lies in bank group x mod 8 of the rows' storage, so
-// the pairs fall into 8 classes; in each they are ranked by entry count (most first) and slot r takes ranks 4 r
-// to 4 r + 3 of every class, so that the lanes of a quarter-warp store to 8 different bank groups and a slot's
-// pairs have similar counts.
+// Gridding runs of the kernels that walk cell pairs (here and in the two-pass 512 x 512 form): an ng x ng grid in
+// rounds of `rows` rows (a round's place of cell (x, y) is stride (y mod rows) + x), each shared out to `warps`
+// warps (at most 16); an antenna's voltage is a shared-memory word of 128 / per bytes.  The 16-byte word of (x, y),
+// y even, lies in bank group x mod 8, so a round's pairs fall into 8 classes; in each they are ranked by entry count
+// (most first) and slot r takes ranks 4 r to 4 r + 3 of every class, so that the lanes of a quarter-warp store to 8
+// different bank groups and a slot's pairs have similar counts.
+void pair_run_tables(int ng, int rows, int stride, int warps, int per, const std::vector<int>& cptr, const std::vector<int2>& cent,
+                     const std::vector<float>& cwim, std::vector<int4>& run, std::vector<float2>& w, std::vector<float2>& wim,
+                     std::vector<uint32_t>& key, std::vector<uint16_t>& empty) {
+    constexpr int MAXW = 16;
+    const int NG = ng, NSLOT = rows * ng / 64;
+    struct Entry { int ant; float2 w, wi; };
+    struct Pair { int off; std::vector<Entry> e; };
+    const float2 none = make_float2(0.f, 0.f);
+    run.clear();
+    for (int rb = 0; rb < ng / rows; ++rb) {
+        std::vector<Pair> pr(rows * NG / 2);
+        std::vector<std::vector<int>> cls(8);
+        for (int yp = 0; yp < rows / 2; ++yp)
+            for (int x = 0; x < NG; ++x) {
+                const int c = (rb * rows + 2 * yp) * NG + x;
+                Pair& p = pr[yp * NG + x];
+                p.off = 2 * yp * stride + x;
+                int i = cptr[c], j = cptr[c + NG];           // both in antenna order
+                while (i < cptr[c + 1] || j < cptr[c + NG + 1]) {
+                    const int ai = i < cptr[c + 1] ? cent[i].y : 1 << 30, aj = j < cptr[c + NG + 1] ? cent[j].y : 1 << 30;
+                    Entry e{std::min(ai, aj), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+                    if (ai == e.ant) {
+                        std::memcpy(&e.w.x, &cent[i].x, sizeof(float));
+                        e.wi.x = cwim[i++];
+                    }
+                    if (aj == e.ant) {
+                        std::memcpy(&e.w.y, &cent[j].x, sizeof(float));
+                        e.wi.y = cwim[j++];
+                    }
+                    p.e.push_back(e);
+                }
+                cls[x & 7].push_back(yp * NG + x);
+            }
+        for (auto& c : cls)
+            std::stable_sort(c.begin(), c.end(), [&](int u, int v) { return pr[u].e.size() > pr[v].e.size(); });
+        std::vector<int> steps(NSLOT, 0), order(NSLOT);
+        for (int r = 0; r < NSLOT; ++r) {
+            order[r] = r;
+            for (auto& c : cls) steps[r] = std::max(steps[r], (int)pr[c[4 * r]].e.size());
+        }
+        std::stable_sort(order.begin(), order.end(), [&](int u, int v) { return steps[u] > steps[v]; });
+        // slots to the warps, heaviest first, each to the warp with the fewest steps (one for a slot that no antenna
+        // reaches: its zeros are stored all the same)
+        std::vector<int> mine[MAXW];
+        int load[MAXW] = {};
+        for (int r : order) {
+            const int wp = (int)(std::min_element(load, load + warps) - load);
+            mine[wp].push_back(r);
+            load[wp] += std::max(1, steps[r]);
+        }
+        for (int wp = 0; wp < warps; ++wp) {
+            run.push_back(int4{(int)key.size(), 0, (int)empty.size(), 0});
+            int4& me = run.back();
+            for (int r : mine[wp]) {
+                std::vector<Entry> rem[32];
+                uint32_t off[32];
+                for (int l = 0; l < 32; ++l) {
+                    const Pair& p = pr[cls[l & 7][4 * r + l / 8]];
+                    rem[l] = p.e;
+                    off[l] = (uint32_t)p.off;
+                    if (steps[r] == 0) empty.push_back((uint16_t)p.off);
+                }
+                if (steps[r] == 0) ++me.w;
+                for (int k = 0; k < steps[r]; ++k) {
+                    int pick[32], banks[4][16] = {}, some = -1;
+                    for (int l = 0; l < 32; ++l) {
+                        pick[l] = -1;
+                        if (rem[l].empty()) continue;
+                        // of the lane's remaining entries, one whose bank the lanes that load together use least at this step
+                        pick[l] = 0;
+                        for (int j = 1; j < (int)rem[l].size(); ++j)
+                            if (banks[l / per][rem[l][j].ant & (per - 1)] < banks[l / per][rem[l][pick[l]].ant & (per - 1)]) pick[l] = j;
+                        some = rem[l][pick[l]].ant;
+                        ++banks[l / per][some & (per - 1)];
+                    }
+                    for (int l = 0; l < 32; ++l) {
+                        // past its list a lane gets zero weights and an antenna that another lane reads at this step
+                        const bool has = pick[l] >= 0;
+                        const Entry x = has ? rem[l][pick[l]] : Entry{some, none, none};
+                        w.push_back(x.w);
+                        wim.push_back(x.wi);
+                        key.push_back((uint32_t)x.ant | (k + 1 == steps[r] ? off[l] << 16 | kGridLast : 0u));
+                        if (has) rem[l].erase(rem[l].begin() + pick[l]);
+                    }
+                }
+                me.y += steps[r];
+            }
+            for (; me.y % kGridAhead != 0; ++me.y)
+                for (int l = 0; l < 32; ++l) {
+                    w.push_back(none);
+                    wim.push_back(none);
+                    key.push_back((uint32_t)cent[0].y);        // a run that is not empty has entries
+                }
+        }
+    }
+}
+
 void half256_tables(const std::vector<int>& cptr, const std::vector<int2>& cent, const std::vector<float>& cwim,
                     std::vector<int4>& run, std::vector<float2>& w, std::vector<float2>& wim,
                     std::vector<uint32_t>& key, std::vector<uint16_t>& empty) {
-    using namespace half256;
-    struct Entry { int ant; float2 w, wi; };
-    struct Pair { int off; std::vector<Entry> e; };
-    std::vector<Pair> pr(NG * NG / 2);
-    std::vector<std::vector<int>> cls(8);
-    for (int yp = 0; yp < NG / 2; ++yp)
-        for (int x = 0; x < NG; ++x) {
-            const int c = 2 * yp * NG + x;
-            Pair& p = pr[yp * NG + x];
-            p.off = 2 * yp * RBS + x;
-            int i = cptr[c], j = cptr[c + NG];           // both in antenna order
-            while (i < cptr[c + 1] || j < cptr[c + NG + 1]) {
-                const int ai = i < cptr[c + 1] ? cent[i].y : 1 << 30, aj = j < cptr[c + NG + 1] ? cent[j].y : 1 << 30;
-                Entry e{std::min(ai, aj), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-                if (ai == e.ant) {
-                    std::memcpy(&e.w.x, &cent[i].x, sizeof(float));
-                    e.wi.x = cwim[i++];
-                }
-                if (aj == e.ant) {
-                    std::memcpy(&e.w.y, &cent[j].x, sizeof(float));
-                    e.wi.y = cwim[j++];
-                }
-                p.e.push_back(e);
-            }
-            cls[x & 7].push_back(yp * NG + x);
-        }
-    for (auto& c : cls)
-        std::stable_sort(c.begin(), c.end(), [&](int u, int v) { return pr[u].e.size() > pr[v].e.size(); });
-    std::vector<int> steps(NSLOT, 0), order(NSLOT);
-    for (int r = 0; r < NSLOT; ++r) {
-        order[r] = r;
-        for (auto& c : cls) steps[r] = std::max(steps[r], (int)pr[c[4 * r]].e.size());
-    }
-    std::stable_sort(order.begin(), order.end(), [&](int u, int v) { return steps[u] > steps[v]; });
-    // slots to the warps, heaviest first, each to the warp with the fewest steps (one for a slot that no antenna
-    // reaches: its zeros are stored all the same)
-    constexpr int NWARP = NT / 32;
-    std::vector<int> mine[NWARP];
-    int load[NWARP] = {};
-    for (int r : order) {
-        const int wp = (int)(std::min_element(load, load + NWARP) - load);
-        mine[wp].push_back(r);
-        load[wp] += std::max(1, steps[r]);
-    }
-    run.assign(NWARP, int4{0, 0, 0, 0});
-    const float2 none = make_float2(0.f, 0.f);
-    for (int wp = 0; wp < NWARP; ++wp) {
-        run[wp].x = (int)key.size();
-        run[wp].z = (int)empty.size();
-        for (int r : mine[wp]) {
-            std::vector<Entry> rem[32];
-            uint32_t off[32];
-            for (int l = 0; l < 32; ++l) {
-                const Pair& p = pr[cls[l & 7][4 * r + l / 8]];
-                rem[l] = p.e;
-                off[l] = (uint32_t)p.off;
-                if (steps[r] == 0) empty.push_back((uint16_t)p.off);
-            }
-            if (steps[r] == 0) ++run[wp].w;
-            for (int k = 0; k < steps[r]; ++k) {
-                int pick[32], banks[2][16] = {}, some = -1;
-                for (int l = 0; l < 32; ++l) {
-                    pick[l] = -1;
-                    if (rem[l].empty()) continue;
-                    // of the lane's remaining entries, one whose 8-byte bank its half-warp uses least at this step
-                    pick[l] = 0;
-                    for (int j = 1; j < (int)rem[l].size(); ++j)
-                        if (banks[l / 16][rem[l][j].ant & 15] < banks[l / 16][rem[l][pick[l]].ant & 15]) pick[l] = j;
-                    some = rem[l][pick[l]].ant;
-                    ++banks[l / 16][some & 15];
-                }
-                for (int l = 0; l < 32; ++l) {
-                    // past its list a lane gets zero weights and an antenna that another lane reads at this step
-                    const bool has = pick[l] >= 0;
-                    const Entry x = has ? rem[l][pick[l]] : Entry{some, none, none};
-                    w.push_back(x.w);
-                    wim.push_back(x.wi);
-                    key.push_back((uint32_t)x.ant | (k + 1 == steps[r] ? off[l] << 16 | kLast : 0u));
-                    if (has) rem[l].erase(rem[l].begin() + pick[l]);
-                }
-            }
-            run[wp].y += steps[r];
-        }
-        for (; run[wp].y % kAhead != 0; ++run[wp].y)
-            for (int l = 0; l < 32; ++l) {
-                w.push_back(none);
-                wim.push_back(none);
-                key.push_back((uint32_t)cent[0].y);        // a run that is not empty has entries
-            }
-    }
+    pair_run_tables(half256::NG, half256::NG, half256::RBS, 16, 16, cptr, cent, cwim, run, w, wim, key, empty);
 }
 
 bool half256_fits(int n_ant, size_t smem_optin) {
