@@ -17,17 +17,19 @@
 // MMAs with N = 256 per 16 samples give D = R_a [R_b; I_b]^T + I_a [I_b; -R_b]^T:
 // Re V in columns 0..127 and -Im V in 128..255.  The CTA's warps have three roles, handing work
 // over through mbarriers only (no CTA-wide barrier inside the loop):
-//   - two sets of 8 decode warps take alternate chunks and convert their voltages (loaded into
-//     registers two of the set's chunks ahead) into one stage of a 5-stage ring; each warp fences
+//   - sets of 8 decode warps (two, or three for voltages read one by one) take the chunks in turn and
+//     convert their voltages (loaded into registers three of the set's chunks ahead) into one
+//     stage of a 3-stage ring; each warp fences
 //     its stores for the tensor cores and arrives on the stage's full barrier, and refills a
 //     stage after the MMAs that read it have completed (the stage's empty barrier, signalled by
 //     tcgen05.commit);
 //   - one thread of the MMA warp issues the 4 MMAs (M = 128, N = 256, K = 16) of a chunk into one
 //     of two TMEM accumulator buffers (all 512 columns), commits each chunk to its stage's empty
 //     barrier and a unit's last chunk to the buffer's full barrier;
-//   - 4 epilogue warps (one per TMEM lane quarter) read a finished buffer (tcgen05.ld), scale
-//     by g_a conj(g_b) / T, write the block (16-byte stores along rows) and, off the diagonal,
-//     its mirrored conjugate, then release the buffer, while the next unit fills the other one.
+//   - 8 (or 4) epilogue warps read a finished buffer (tcgen05.ld), scale by g_a conj(g_b) / T with
+//     the gains in shared memory, write the block (16 adjacent elements at a time) and, off the
+//     diagonal, its mirrored conjugate, then release the buffer, while the next unit fills the
+//     other one.
 // Every wait is bounded by the plan's try count and taken by a whole warp; on a timeout the role
 // stops, the CTA sets the correlator-timeout bit of the plan's status word and writes NaN into
 // its first output element; the MMA warp waits (full limit) for the MMAs it issued before the
@@ -37,6 +39,15 @@
 // of each of its 8 samples with 4-byte loads (a warp reads whole 128-byte rows), transposes the
 // 4 x 4 byte blocks with byte permutes and converts each 4 samples of an antenna with two
 // permute + packed-subtraction pairs per plane.  Other voltages are read one by one.
+//
+// Bound by the latency of the decode's loads and of the epilogue's stores (the products alone take 43 us of
+// 115 in the first case below) and, where the units do not divide over the SMs, by the last of them (768 units on
+// 152 SMs: six turns for 5.05).  A copy of the kernel without the epilogue's 15 / 16 took 72 of 105 us: its
+// column gains came from L2 one by one, because the stages leave a few KB of the SM to L1.  Measured before and
+// now (us; antennas x samples x (channel, pol)): 4+4-bit 256 x 1024 x 256: 140 and 116; 256 x 64 x 256: 88 and 44;
+// 256 x 1024 x 1: 37 and 29; 1024 x 1024 x 16: 111 and 95; 254 x 1024 x 256: 287 and 254; FP16 256 x 1024 x 256: 292
+// and 192.
+#include <algorithm>
 #include <cuda_fp16.h>
 #include <cstdint>
 #include "moff_common.cuh"
@@ -46,11 +57,6 @@ namespace epic {
 namespace xe {
 using namespace tc;
 
-constexpr int NDS = 3;                      // decode warp sets, taking alternate chunks
-constexpr int NDW = 8 * NDS;                // decode warps (a set's tile mappings take 256 threads)
-constexpr int NEW = 4;                      // epilogue warps, one per TMEM lane quarter
-constexpr int MMA_WARP = NDW;               // the warp whose first thread issues the MMAs
-constexpr int NT = 32 * (NDW + 1 + NEW);    // one CTA per SM
 constexpr int TC = 32;                      // samples per K chunk (K = 32: one real plane per operand row)
 // K-major FP16 planes without swizzle: 8 x 8 core matrices of 128 bytes, a row group of 8 rows
 // holding the chunk's 4 core matrices along K
@@ -59,12 +65,30 @@ constexpr int kPlaneBytes = 16 * kRowGroupBytes;       // 128 rows x 32 samples 
 constexpr int kBTileBytes = 3 * kPlaneBytes;           // [Re_b; Im_b; -Re_b]: 384 rows
 constexpr int kATileBytes = 2 * kPlaneBytes;           // [Re_a; Im_a]
 constexpr int kStageBytes = kBTileBytes + kATileBytes; // 40 KB
-constexpr int NSTAGE = 5;
-// mbarriers: stage full [NSTAGE], stage empty [NSTAGE], accumulator full [2], accumulator
-// empty [2], drain
-constexpr int N_MBAR = 2 * NSTAGE + 5;
+// an epilogue warp's 32 rows x 16 columns, rows 144 bytes apart (16-byte accesses of 8 lanes hit all 32 banks)
+constexpr int kRowStride = 18;
 
-constexpr size_t smem_bytes() { return (size_t)NSTAGE * kStageBytes + 8 * N_MBAR + 16; }
+// The roles of a CTA's warps (one CTA per SM).  Measured (us, 256 antennas, 256 (channel, pol), 4+4-bit voltages of
+// 1,024 and of 64 samples; sets, epilogue warps, stages): 2, 8, 3: 116 and 44; 3, 4, 3: 113 and 61; 2, 8, 4: 121 and
+// 45; 3, 4, 5: 119 and 61; 1, 8, 4: 193 and 54.  More stages leave less L1 for the loads in flight: FP16 voltages of
+// 1,024 samples (read one by one, so with three sets) take 192 with 3 stages and 257 with 5.
+template <bool WIDE>
+struct Roles {
+    static constexpr int NDS = WIDE ? 2 : 3;                // decode warp sets, taking alternate chunks
+    static constexpr int NDW = 8 * NDS;                     // decode warps (a set's tile mappings take 256 threads)
+    static constexpr int NEW = WIDE ? 8 : 4;                // epilogue warps, NEW / 4 per TMEM lane quarter
+    static constexpr int MMA_WARP = NDW;                    // the warp whose first thread issues the MMAs
+    static constexpr int NT = 32 * (NDW + 1 + NEW);
+    static constexpr int NSTAGE = 3;
+    // a set waits for its stage's last use but one at most: with fewer stages than sets it could take the phase
+    // before for the one it waits for
+    static_assert(NSTAGE >= NDS, "stages");
+    // mbarriers: stage full [NSTAGE], stage empty [NSTAGE], accumulator full [2], accumulator
+    // empty [2], drain
+    static constexpr int N_MBAR = 2 * NSTAGE + 5;
+    static constexpr size_t kSmem = (size_t)NSTAGE * kStageBytes + (size_t)NEW * (32 * kRowStride + 128) * sizeof(float2) +
+                                    8 * N_MBAR + 16;
+};
 
 // One voltage as an FP16 (re, im) pair (half2 bits).  FP16 input is already the pair.  A
 // 4+4-bit byte holds two 4-bit two's-complement values (re in the high nibble); XOR with 8 biases
@@ -98,12 +122,16 @@ __device__ __forceinline__ void unit_coords(int u, int nab, int& cp, int& ab, in
 }
 
 template <int VDT, bool WIDE>
-__global__ void __launch_bounds__(NT, 1) xeng_kernel(const XengArgs a) {
+__global__ void __launch_bounds__(Roles<WIDE>::NT, 1) xeng_kernel(const XengArgs a) {
+    using W = Roles<WIDE>;
+    constexpr int NDS = W::NDS, NDW = W::NDW, NEW = W::NEW, MMA_WARP = W::MMA_WARP, NSTAGE = W::NSTAGE, N_MBAR = W::N_MBAR;
     static_assert(!WIDE || VDT == 2, "the wide loads are for 4+4-bit voltages");
     using VT = typename Volt<VDT>::T;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* sT = smem_raw;                                               // [NSTAGE] stages
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(sT + (size_t)NSTAGE * kStageBytes);   // [N_MBAR]
+    float2* sRows = reinterpret_cast<float2*>(sT + (size_t)NSTAGE * kStageBytes);      // [NEW][32][kRowStride]
+    float2* sGain = sRows + NEW * 32 * kRowStride;                                     // [NEW][128]
+    uint64_t* mbar = reinterpret_cast<uint64_t*>(sGain + NEW * 128);                  // [N_MBAR]
     uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + N_MBAR);
     int* s_fail = reinterpret_cast<int*>(tslot + 1);
 
@@ -195,8 +223,8 @@ __global__ void __launch_bounds__(NT, 1) xeng_kernel(const XengArgs a) {
                                         __byte_perm(x[4], x[5], 0x7632), __byte_perm(x[6], x[7], 0x7632));
             put_planes(tile, i, re, im, neg);
         };
-        // raw words of this thread's 8 samples (fast path: byte i = antenna 4 l + i), two chunks
-        uint32_t rw0[8], rw1[8];
+        // raw words of this thread's 8 samples (fast path: byte i = antenna 4 l + i), three chunks
+        uint32_t rw0[8], rw1[8], rw2[8];
         int lu = beg, lkc = 0, lcp = 0, lab = 0, lbb = 0;                       // load cursor
         advance(lu, lkc, dset);
         if (lu < end) unit_coords(lu, nab, lcp, lab, lbb);
@@ -274,45 +302,40 @@ __global__ void __launch_bounds__(NT, 1) xeng_kernel(const XengArgs a) {
         if constexpr (WIDE) {
             fast_load(rw0);
             fast_load(rw1);
+            fast_load(rw2);
         }
         bool failed = false;
         int cu = beg, ckc = 0, ccp = 0, cab = 0, cbb = 0;                       // decode cursor
         advance(cu, ckc, dset);
         if (cu < end) unit_coords(cu, nab, ccp, cab, cbb);
-        for (int i = 0; cu < end; ++i) {
+        auto one = [&](uint32_t (&rw)[8]) -> bool {
+            if (cu >= end) return false;
             const int g = (cu - beg) * n_chunks + ckc;
             const int s = g % NSTAGE;
             // the stage is free once the MMAs of its previous chunk have completed
             if (g >= NSTAGE && !warp_wait(mb_empty(s), (g / NSTAGE - 1) & 1)) {
                 failed = true;
-                break;
+                return false;
             }
             const bool diag = cab == cbb;
             unsigned char* st = sT + (size_t)s * kStageBytes;
             if (bside || !diag) {
                 unsigned char* tile = bside ? st : st + kBTileBytes;
-                if constexpr (WIDE) {
-                    if ((i & 1) == 0)
-                        fast_decode(rw0, tile);
-                    else
-                        fast_decode(rw1, tile);
-                } else {
-                    slow_decode(ccp, bside ? cbb : cab, ckc, tile);
-                }
+                if constexpr (WIDE) fast_decode(rw, tile);
+                else slow_decode(ccp, bside ? cbb : cab, ckc, tile);
             }
             // this warp's stores, visible to the tensor cores, then its arrival
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(mb_full(s));
-            // the set's chunk after next into the register set just decoded
-            if constexpr (WIDE) {
-                if ((i & 1) == 0)
-                    fast_load(rw0);
-                else
-                    fast_load(rw1);
-            }
+            // the set's third chunk from here into the registers just decoded
+            if constexpr (WIDE) fast_load(rw);
             if (advance(cu, ckc, NDS) && cu < end) unit_coords(cu, nab, ccp, cab, cbb);
-        }
+            return true;
+        };
+        // unrolled over the register sets (chosen by a branch, the sets cost 6 % of the call's time)
+#pragma unroll 1
+        while (one(rw0) && one(rw1) && one(rw2)) {}
         if (failed) *s_fail = 1;
     } else if (warp == MMA_WARP) {
         // ---------------- MMA warp: per K step of 16 samples two MMAs (M = 128, N = 256) ----
@@ -373,55 +396,78 @@ __global__ void __launch_bounds__(NT, 1) xeng_kernel(const XengArgs a) {
         bool failed = false;
         const int q = warp & 3;                   // TMEM lane quarter this warp may read
         const float inv_t = 1.f / float(T);
+        const int ew = warp - MMA_WARP - 1, c0 = ew / 4 * (512 / NEW);      // its columns: c0 .. + 512 / NEW
+        float2 *rows = sRows + ew * 32 * kRowStride, *gcol = sGain + ew * 128;
         // 16-byte row stores when every row starts on a 16-byte boundary
         const bool vec = (A % 2 == 0) && ((reinterpret_cast<uintptr_t>(a.vis) & 15) == 0);
         int n = 0;
         for (int u = beg; u < end; ++u, ++n) {
             const int b = n & 1;
-            if (!warp_wait(mb_accf(b), (n >> 1) & 1)) {
-                failed = true;
-                break;
-            }
-            fence_after();
             int cp, ab, bb;
             unit_coords(u, nab, cp, ab, bb);
             const bool diag = ab == bb;
             const int a0 = ab * 128, b0 = bb * 128;
             const int aa = a0 + 32 * q + lane;
             const uint32_t tacc = tmem + 256 * b + ((uint32_t)(32 * q) << 16);
-            const float2 ga = (aa < A && a.gains) ? a.gains[(size_t)cp * A + aa] : make_float2(1.f, 0.f);
+            // the unit's gains while its products are summed: this lane's row, and the columns in shared memory (read
+            // from L2 column by column they were most of the epilogue's time)
+            const float2 one = make_float2(1.f, 0.f), *gn = a.gains ? a.gains + (size_t)cp * A : nullptr;
+            const float2 ga = (gn && aa < A) ? __ldg(gn + aa) : one;
+#pragma unroll
+            for (int i = lane; i < 128; i += 32) gcol[i] = (gn && b0 + i < A) ? __ldg(gn + b0 + i) : one;
+            __syncwarp();
+            if (!warp_wait(mb_accf(b), (n >> 1) & 1)) {
+                failed = true;
+                break;
+            }
+            fence_after();
             float2* out = a.vis + (size_t)cp * A * A;
+            // 16 columns at a time.  A lane holds a row, so the mirrored block is written 32 adjacent elements at a
+            // time, and on the diagonal, where the block is its own mirror, it alone.  Off the diagonal the rows
+            // themselves go through shared memory, to be written 16 adjacent elements at a time.
 #pragma unroll 1
-            for (int c = 0; c < 128; c += 8) {
-                float dr[8], di[8];
-                tld<8>(tacc + c, dr);
-                tld<8>(tacc + 128 + c, di);
-                tld_wait();
-                if (aa < A) {
+            for (int c = c0; c < c0 + 512 / NEW; c += 16) {
+#pragma unroll
+                for (int h = 0; h < 16; h += 8) {
+                    float dr[8], di[8];
+                    tld<8>(tacc + c + h, dr);
+                    tld<8>(tacc + 128 + c + h, di);
+                    tld_wait();
                     float2 v[8];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int bcol = b0 + c + j;
-                        const float2 gb = (a.gains && bcol < A) ? __ldg(a.gains + (size_t)cp * A + bcol)
-                                                                : make_float2(1.f, 0.f);
-                        const float2 w = cmul(ga, make_float2(gb.x, -gb.y));
-                        v[j] = cmul(w, make_float2(dr[j] * inv_t, -di[j] * inv_t));   // D holds -Im V
-                    }
-                    float2* row = out + (size_t)aa * A + b0 + c;
-                    if (vec && b0 + c + 8 <= A) {
-                        float4* r4 = reinterpret_cast<float4*>(row);
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) r4[j] = make_float4(v[2 * j].x, v[2 * j].y, v[2 * j + 1].x, v[2 * j + 1].y);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            if (b0 + c + j < A) row[j] = v[j];
+                    for (int j = 0; j < 8; ++j) {                // D holds -Im V
+                        const float2 gb = gcol[c + h + j];
+                        const float2 w = diag ? cmul(gb, make_float2(ga.x, -ga.y)) : cmul(ga, make_float2(gb.x, -gb.y));
+                        v[j] = cmul(w, make_float2(dr[j] * inv_t, (diag ? di[j] : -di[j]) * inv_t));
+                        if (aa < A && b0 + c + h + j < A)
+                            out[(size_t)(b0 + c + h + j) * A + aa] = make_float2(v[j].x, diag ? v[j].y : -v[j].y);
                     }
                     if (!diag) {
 #pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            if (b0 + c + j < A) out[(size_t)(b0 + c + j) * A + aa] = make_float2(v[j].x, -v[j].y);
+                        for (int j = 0; j < 8; j += 2)
+                            *reinterpret_cast<float4*>(rows + lane * kRowStride + h + j) =
+                                make_float4(v[j].x, v[j].y, v[j + 1].x, v[j + 1].y);
                     }
+                }
+                if (!diag) {
+                    __syncwarp();
+                    const int r0 = a0 + 32 * q;
+                    if (vec && b0 + c + 16 <= A) {
+#pragma unroll
+                        for (int i = 0; i < 32; i += 4) {
+                            const int r = i + (lane >> 3), k = 2 * (lane & 7);
+                            const float4 x = *reinterpret_cast<const float4*>(rows + r * kRowStride + k);
+                            if (r0 + r < A) *reinterpret_cast<float4*>(out + (size_t)(r0 + r) * A + b0 + c + k) = x;
+                        }
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 32; i += 2) {
+                            const int r = i + (lane >> 4), k = lane & 15;
+                            const float2 x = rows[r * kRowStride + k];
+                            if (r0 + r < A && b0 + c + k < A) out[(size_t)(r0 + r) * A + b0 + c + k] = x;
+                        }
+                    }
+                    __syncwarp();
                 }
             }
             // this warp's reads of buffer b are complete: the MMA warp may overwrite it
@@ -756,7 +802,7 @@ cudaError_t launch_fx_image_t(const FxArgs& a, cudaStream_t st) {
 
 }  // namespace xe
 
-size_t xeng_smem_bytes() { return xe::smem_bytes(); }
+size_t xeng_smem_bytes() { return std::max(xe::Roles<false>::kSmem, xe::Roles<true>::kSmem); }
 
 cudaError_t launch_fx_image(int n_pad, const FxArgs& a, cudaStream_t st) {
     if (a.n_cp == 0) return cudaSuccess;
@@ -771,10 +817,10 @@ cudaError_t launch_fx_image(int n_pad, const FxArgs& a, cudaStream_t st) {
 namespace {
 template <int VDT, bool WIDE>
 cudaError_t launch_xeng_t(const XengArgs& a, long long grid, cudaStream_t st) {
-    const size_t smem = xe::smem_bytes();
+    constexpr size_t smem = xe::Roles<WIDE>::kSmem;
     const cudaError_t e = ensure_smem<xe::xeng_kernel<VDT, WIDE>>(smem);
     if (e != cudaSuccess) return e;
-    xe::xeng_kernel<VDT, WIDE><<<(unsigned)grid, xe::NT, smem, st>>>(a);
+    xe::xeng_kernel<VDT, WIDE><<<(unsigned)grid, xe::Roles<WIDE>::NT, smem, st>>>(a);
     return cudaGetLastError();
 }
 }  // namespace

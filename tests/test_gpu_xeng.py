@@ -254,3 +254,18 @@ def test_gpu_fx_image_folded_pairs(epic, n_cp, n_ant):
     for c in range(n_cp):
         want = (K * (vis[c, 0].astype(np.complex64).astype(np.complex128) @ K.conj())).sum(0).real.reshape(n_pad, n_pad)
         assert np.linalg.norm(img[c, 0] - want) < 1e-5 * np.linalg.norm(want), c
+
+
+@pytest.mark.parametrize("n_ant, n_time, n_cp, vdtype, gains", [
+    (129, 33, 1, "ci4", True),      # a one-antenna tail column block, rows of odd length: 8-byte row stores
+    (146, 5, 2, "f16", True),       # an 18-antenna tail: one full group of 16 columns and 2 of the next
+    (256, 96, 153, "ci4", False),   # 459 units: buffers and gain slots reused, no gains; three chunks
+    (260, 97, 2, "ci4", True),      # a 4-antenna tail block, four chunks with one sample in the last
+])
+def test_epilogue_blocks(epic, n_ant, n_time, n_cp, vdtype, gains):
+    """Blocks written row by row through shared memory and mirrored, at ragged column groups, with and
+    without gains, and chunk counts around the decode sets' turns.  Against the oracle in float64 (TOL)."""
+    wl = _small(n_ant, n_time, n_cp, 1, vdtype, seed=n_ant)
+    g = synth.random_gains(np.random.default_rng(n_ant), (n_cp, 1, n_ant)) if gains else None
+    _, vis = run(epic, wl, g)
+    check(vis, wl, g, "A=%d" % n_ant)
