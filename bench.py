@@ -34,23 +34,27 @@ SM_MAX_MHZ = 2070.0
 # dram__bytes_read.sum + dram__bytes_write.sum per launch on this workload, from ncu captures
 # of the 8-channel case (16,384 images) scaled by the units per launch (x16); None until
 # captured for the current kernel.  Forward FFT kernel: 6.46 MB per capture; tensor-core
-# DFT-GEMM kernel: 6.57 MB per capture.
+# DFT-GEMM kernel: 6.44 MB per capture.
 FWD_TRAFFIC_BYTES = 103.4e6
-DG_TRAFFIC_BYTES = 105.2e6
+DG_TRAFFIC_BYTES = 103.1e6
 # F-engine on the headline shapes (one full launch captured: 67.1 MB read, 207.1 MB written;
 # the last spectra written are still in L2 when the kernel ends)
 FENGINE_TRAFFIC_BYTES = 274.2e6
-# X-engine on the headline workload (one full launch captured: 79.6 MB read, 77.3 MB written)
-XENG_TRAFFIC_BYTES = 156.9e6
+# X-engine on the headline workload (one full launch captured: 81.5 MB read, 77.8 MB written)
+XENG_TRAFFIC_BYTES = 159.3e6
 # Work of the tensor-core DFT form per 128 x 128 image.  Algorithmic: the pruned transform as
 # two complex matrix products, each four real products -- stage 1 X = W E (128 x 64 outputs,
-# K = 64), stage 2 F = X W^T (128 x 128 outputs, K = 64): 12.58 MFLOP.  Executed: every real
-# product as three FP16 products (hi*hi + hi*lo + lo*hi) to reach FP32 accuracy: 3x that.
+# K = 64), stage 2 F = X W^T (128 x 128 outputs, K = 64): 12.58 MFLOP; with every real product as
+# three FP16 products (hi*hi + hi*lo + lo*hi), to reach FP32 accuracy, 3x that.  Executed: the
+# frequencies in pairs halve the products: 18.87 MFLOP (36 MMAs of 128 x 128 x 16), and 6.29
+# MFLOP in the reduced-precision form (one FP16 product each).
 DG_ALG_FLOP_PER_IMAGE = 4 * 2.0 * 128 * 64 * 64 + 4 * 2.0 * 128 * 128 * 64
 DG_FLOP_PER_IMAGE = 3 * DG_ALG_FLOP_PER_IMAGE
+DG_EXEC_FLOP_PER_IMAGE = DG_FLOP_PER_IMAGE / 2
+DG_LP_FLOP_PER_IMAGE = DG_ALG_FLOP_PER_IMAGE / 2
 # sm__pipe_tensor_cycles_active of the tensor-core kernel in its latest small-case ncu capture
 # (8 channels x 2 pols x 1024 samples, one launch)
-DG_TENSOR_ACTIVE_NCU = 0.591
+DG_TENSOR_ACTIVE_NCU = 0.519
 # standalone gridder: 479.8 MB per capture launch (1,024 of the 16,384 units), scaled x16
 GRID_TRAFFIC_BYTES = 7.677e9
 MEASURED_PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
@@ -802,9 +806,9 @@ def run_xpol(args):
     chosen = min(ok, key=lambda k: forms[k]["ms_per_step"])
     f = forms[chosen]
     if chosen == "fp16x3_dftgemm":
-        roof = tensor_roofline(DG_ALG_FLOP_PER_IMAGE * T * C * 4, DG_FLOP_PER_IMAGE * T * C * 4, f["kernel_ms"],
+        roof = tensor_roofline(DG_ALG_FLOP_PER_IMAGE * T * C * 4, DG_EXEC_FLOP_PER_IMAGE * T * C * 4, f["kernel_ms"],
                                f["clocks"], flop_basis="per virtual-pol image as the headline (pruned DFT as "
-                                                       "real products; executed: 3 FP16 products each), "
+                                                       "real products; executed: half of them, 3 FP16 products each), "
                                                        "4 per channel-sample")
     else:
         flops = workload_algorithmic_flops(wl, plan.info["nnz"]) * T * C * 4
@@ -1310,24 +1314,23 @@ def main():
     chosen = min(ok, key=lambda k: forms[k]["ms_per_step"])
     f = forms[chosen]
     if chosen == "fp16x3_dftgemm":
-        roof = tensor_roofline(DG_ALG_FLOP_PER_IMAGE * T * C * P, DG_FLOP_PER_IMAGE * T * C * P, f["kernel_ms"],
+        roof = tensor_roofline(DG_ALG_FLOP_PER_IMAGE * T * C * P, DG_EXEC_FLOP_PER_IMAGE * T * C * P, f["kernel_ms"],
                                f["clocks"], traffic=DG_TRAFFIC_BYTES, ncu_active=DG_TENSOR_ACTIVE_NCU,
                                flop_basis="algorithmic: the pruned 128 x 128 DFT of each image as real products, "
                                           "%.2f MFLOP (stage 1 128x64 outputs, stage 2 128x128, K = 64); executed: "
-                                          "3 FP16 products (hi*hi + hi*lo + lo*hi) per real product, %.2f MFLOP"
-                                          % (DG_ALG_FLOP_PER_IMAGE / 1e6, DG_FLOP_PER_IMAGE / 1e6))
+                                          "half of them (frequencies in pairs), 3 FP16 products (hi*hi + hi*lo + lo*hi) each, %.2f MFLOP"
+                                          % (DG_ALG_FLOP_PER_IMAGE / 1e6, DG_EXEC_FLOP_PER_IMAGE / 1e6))
     else:
         roof = alu_roofline(fft_flops, f["kernel_ms"], n_sm, f["clocks"], traffic=FWD_TRAFFIC_BYTES)
     # the plain FP32 form's own roofline, whichever form is chosen
     fft_roof = alu_roofline(fft_flops, forms["fp32_fft"]["kernel_ms"], n_sm, forms["fp32_fft"]["clocks"],
                             traffic=FWD_TRAFFIC_BYTES)
-    # the reduced-precision tensor-core form: one FP16 product per real product (executed =
-    # algorithmic work), reported with its own error (its bound is 3e-3, not the FP32 path's)
+    # the reduced-precision tensor-core form: one FP16 product per real product, reported with its own error (its bound is 3e-3, not the FP32 path's)
     lp = forms["fp16_dftgemm"]
-    lp["roofline"] = tensor_roofline(DG_ALG_FLOP_PER_IMAGE * T * C * P, DG_ALG_FLOP_PER_IMAGE * T * C * P,
+    lp["roofline"] = tensor_roofline(DG_ALG_FLOP_PER_IMAGE * T * C * P, DG_LP_FLOP_PER_IMAGE * T * C * P,
                                      lp["kernel_ms"], lp["clocks"],
-                                     flop_basis="the pruned 128 x 128 DFT as real products, 12.58 MFLOP per image, "
-                                                "each one FP16 product")
+                                     flop_basis="the pruned 128 x 128 DFT as real products, 12.58 MFLOP per image; "
+                                                "executed: half of them (frequencies in pairs), one FP16 product each")
     # the standalone gridder (epic_grid) on the same resident voltages: the gridded fields of all
     # 262,144 samples written to HBM, against the measured copy bandwidth
     grid = measure_gridder(wl, plan, volt, dev, args.steps, args.warmup, world, rank, flush,

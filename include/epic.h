@@ -112,8 +112,9 @@ epic_status epic_create(epic_plan **plan, int n_ant, const double *pos_xy,
  * DFT matrix W[k][n] = exp(+2 pi i n k / N_p) on the tensor cores: every operand is split into
  * two FP16 numbers (hi + lo) and each real product is accumulated as hi*hi + hi*lo + lo*hi in
  * FP32 (per image the gridded field is scaled by a power of two to keep the operands in range).
- * It is available for n_pad == 128 (up to about 2,400 antennas: the kernel keeps four
- * per-antenna arrays in shared memory beside the operand tables; 1,900 for epic_image_xpol) and
+ * It is available for n_pad == 128 (up to about 2,400 antennas, which have to fit shared memory
+ * beside the operand tables; 1,900 for epic_image_xpol; frequencies in pairs +-(k + 1/2), half the
+ * products of the dense form) and
  * for n_pad == 256 (up to about 1,860 antennas; two CTAs per image, each computing half of the
  * image rows, the operand tables streamed from global memory; no cross-polarisation form);
  * otherwise EPIC_EUNSUPPORTED.  EPIC_XFORM_DFTGEMM_FP16 (n_pad == 128, single polarisation
@@ -121,12 +122,13 @@ epic_status epic_create(epic_plan **plan, int n_ant, const double *pos_xy,
  * FP16-rounded calibrated voltages and sums in FP32, and each real product of the transform is
  * one FP16 product with FP32 accumulation (no lo parts): about a third of the tensor work, with
  * an error of about 1e-3 relative L2 against the exact image instead of about 1e-6.  The first
- * call with a tensor-core form uploads the plan's DFT operand tables (64 KB for n_pad 128,
+ * call with a tensor-core form uploads the plan's DFT operand tables (34 KB for n_pad 128,
  * 256 KB for 256).  EPIC_XFORM_FFT_TWOPASS (n_pad == 512) computes the same FP32 transform as the
  * default form in two passes over every SM instead of one 16-CTA cluster per image (only one
- * such cluster fits a GPC): the row pass writes each sample's row-transformed grid (1 MB) to a
- * scratch buffer the plan allocates on the first call (4 x SMs samples, about 608 MB on 152
- * SMs), the column pass reads it back; no cross-polarisation variant.
+ * such cluster fits a GPC), two samples or two columns at a time: the row pass writes each
+ * sample's row-transformed grid (1 MB) to a scratch buffer the plan allocates on the first call
+ * (4 x SMs samples, about 608 MB on 152 SMs), the column pass reads it back; no
+ * cross-polarisation variant.
  * EPIC_XFORM_DFTGEMM_FP16_GRID (n_pad == 256, single polarisation products only) grids with FP16
  * operands -- each weight and each calibrated voltage rounded to FP16 (normal FP16 range: about
  * 6e-5 to 65504 in magnitude), each product exact in FP32, the cells' sums in FP32 -- and then
