@@ -14,7 +14,8 @@
 // pol); one persistent CTA per SM takes a contiguous range of units, K walked in chunks of 32
 // samples.  A chunk's operands are K-major FP16 planes: the B tile [R_b; I_b; -R_b] (384 rows)
 // and the A tile [R_a; I_a] (a diagonal unit takes its A planes from the B tile), so that two
-// MMAs with N = 256 per 16 samples give D = R_a [R_b; I_b]^T + I_a [I_b; -R_b]^T:
+// MMAs with N = 256 per 16 samples give D = R_a [R_b; I_b]^T + I_a [I_b; -R_b]^T (without the plane -R_b
+// where voltages are read one by one: two MMAs of N = 128, one with its A operand negated, for the second):
 // Re V in columns 0..127 and -Im V in 128..255.  The CTA's warps have three roles, handing work
 // over through mbarriers only (no CTA-wide barrier inside the loop):
 //   - sets of 8 decode warps (two, or three for voltages read one by one) take the chunks in turn and
@@ -23,7 +24,7 @@
 //     its stores for the tensor cores and arrives on the stage's full barrier, and refills a
 //     stage after the MMAs that read it have completed (the stage's empty barrier, signalled by
 //     tcgen05.commit);
-//   - one thread of the MMA warp issues the 4 MMAs (M = 128, N = 256, K = 16) of a chunk into one
+//   - one thread of the MMA warp issues the MMAs (M = 128, K = 16) of a chunk into one
 //     of two TMEM accumulator buffers (all 512 columns), commits each chunk to its stage's empty
 //     barrier and a unit's last chunk to the buffer's full barrier;
 //   - 8 (or 4) epilogue warps read a finished buffer (tcgen05.ld), scale by g_a conj(g_b) / T with
@@ -45,8 +46,8 @@
 // 152 SMs: six turns for 5.05).  A copy of the kernel without the epilogue's 15 / 16 took 72 of 105 us: its
 // column gains came from L2 one by one, because the stages leave a few KB of the SM to L1.  Measured before and
 // now (us; antennas x samples x (channel, pol)): 4+4-bit 256 x 1024 x 256: 140 and 116; 256 x 64 x 256: 88 and 44;
-// 256 x 1024 x 1: 37 and 29; 1024 x 1024 x 16: 111 and 95; 254 x 1024 x 256: 287 and 254; FP16 256 x 1024 x 256: 292
-// and 192.
+// 256 x 1024 x 1: 37 and 29; 1024 x 1024 x 16: 111 and 95; 254 x 1024 x 256: 287 and 239; FP16 256 x 1024 x 256: 292
+// and 182.
 #include <algorithm>
 #include <cuda_fp16.h>
 #include <cstdint>
@@ -62,9 +63,8 @@ constexpr int TC = 32;                      // samples per K chunk (K = 32: one 
 // holding the chunk's 4 core matrices along K
 constexpr int kRowGroupBytes = 4 * 128;
 constexpr int kPlaneBytes = 16 * kRowGroupBytes;       // 128 rows x 32 samples (8 KB)
-constexpr int kBTileBytes = 3 * kPlaneBytes;           // [Re_b; Im_b; -Re_b]: 384 rows
 constexpr int kATileBytes = 2 * kPlaneBytes;           // [Re_a; Im_a]
-constexpr int kStageBytes = kBTileBytes + kATileBytes; // 40 KB
+constexpr uint32_t kNegA = 1u << 13;                   // instruction descriptor: negate the A operand
 // an epilogue warp's 32 rows x 16 columns, rows 144 bytes apart (16-byte accesses of 8 lanes hit all 32 banks)
 constexpr int kRowStride = 18;
 
@@ -79,6 +79,13 @@ struct Roles {
     static constexpr int NEW = WIDE ? 8 : 4;                // epilogue warps, NEW / 4 per TMEM lane quarter
     static constexpr int MMA_WARP = NDW;                    // the warp whose first thread issues the MMAs
     static constexpr int NT = 32 * (NDW + 1 + NEW);
+    // the B tile with the plane -Re_b, or without: then its product is one MMA of N = 128 more with the A operand
+    // negated.  Without it the decode stores a plane less, and the MMAs read their operands in smaller pieces.
+    // Measured (us, with and without, 256 antennas, 256 (channel, pol), 1,024 samples): 4+4-bit 116.9 and 117.6, one
+    // (channel, pol) 29.2 and 30.0; FP16 192 and 182, 254 antennas of 4+4 bits 254 and 239.
+    static constexpr bool NEG_PLANE = WIDE;
+    static constexpr int kBTileBytes = (NEG_PLANE ? 3 : 2) * kPlaneBytes;   // [Re_b; Im_b; -Re_b] or [Re_b; Im_b]
+    static constexpr int kStageBytes = kBTileBytes + kATileBytes;           // 40 or 32 KB
     static constexpr int NSTAGE = 3;
     // a set waits for its stage's last use but one at most: with fewer stages than sets it could take the phase
     // before for the one it waits for
@@ -125,6 +132,7 @@ template <int VDT, bool WIDE>
 __global__ void __launch_bounds__(Roles<WIDE>::NT, 1) xeng_kernel(const XengArgs a) {
     using W = Roles<WIDE>;
     constexpr int NDS = W::NDS, NDW = W::NDW, NEW = W::NEW, MMA_WARP = W::MMA_WARP, NSTAGE = W::NSTAGE, N_MBAR = W::N_MBAR;
+    constexpr int kBTileBytes = W::kBTileBytes, kStageBytes = W::kStageBytes;
     static_assert(!WIDE || VDT == 2, "the wide loads are for 4+4-bit voltages");
     using VT = typename Volt<VDT>::T;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -211,7 +219,7 @@ __global__ void __launch_bounds__(Roles<WIDE>::NT, 1) xeng_kernel(const XengArgs
         auto put_planes = [&](unsigned char* tile, int i, const uint4& re, const uint4& im, bool neg) {
             *reinterpret_cast<uint4*>(tile + soff[i]) = re;
             *reinterpret_cast<uint4*>(tile + kPlaneBytes + soff[i]) = im;
-            if (neg)
+            if (W::NEG_PLANE && neg)
                 *reinterpret_cast<uint4*>(tile + 2 * kPlaneBytes + soff[i]) =
                     make_uint4(re.x ^ 0x80008000u, re.y ^ 0x80008000u, re.z ^ 0x80008000u, re.w ^ 0x80008000u);
         };
@@ -338,7 +346,7 @@ __global__ void __launch_bounds__(Roles<WIDE>::NT, 1) xeng_kernel(const XengArgs
         while (one(rw0) && one(rw1) && one(rw2)) {}
         if (failed) *s_fail = 1;
     } else if (warp == MMA_WARP) {
-        // ---------------- MMA warp: per K step of 16 samples two MMAs (M = 128, N = 256) ----
+        // ---------------- MMA warp: per K step of 16 samples two MMAs (M = 128, N = 256; or three) ----
         //   D += Re_a [Re_b; Im_b]^T,  D += Im_a [Im_b; -Re_b]^T
         // so that D[:, 0:128] = Re_a Re_b + Im_a Im_b = Re V and D[:, 128:256] = Re_a Im_b - Im_a Re_b
         // = -Im V (summed over the samples); on a diagonal unit the A planes are the B tile's.
@@ -346,7 +354,7 @@ __global__ void __launch_bounds__(Roles<WIDE>::NT, 1) xeng_kernel(const XengArgs
         int g = 0;                                // chunks whose MMAs this warp issued
         int n = 0;                                // units started
         const uint64_t d0 = sdesc(smem_u32(sT), kRowGroupBytes);
-        constexpr uint32_t id = idesc(256);
+        [[maybe_unused]] constexpr uint32_t id = idesc(256), id_half = idesc(128);
         for (int u = beg; u < end && !failed; ++u, ++n) {
             int cp, ab, bb;
             unit_coords(u, nab, cp, ab, bb);
@@ -375,7 +383,12 @@ __global__ void __launch_bounds__(Roles<WIDE>::NT, 1) xeng_kernel(const XengArgs
 #pragma unroll
                     for (int j = 0; j < TC / 16; ++j) {
                         mma_ss(tacc, dA1 + 16 * j, dB1 + 16 * j, id, (kc | j) != 0);
-                        mma_ss(tacc, dA2 + 16 * j, dB2 + 16 * j, id, 1);
+                        if constexpr (W::NEG_PLANE) {
+                            mma_ss(tacc, dA2 + 16 * j, dB2 + 16 * j, id, 1);
+                        } else {
+                            mma_ss(tacc, dA2 + 16 * j, dB2 + 16 * j, id_half, 1);
+                            mma_ss(tacc + 128, dA2 + 16 * j, dB1 + 16 * j, id_half | kNegA, 1);
+                        }
                     }
                     commit(mb_empty(s));
                     if (kc == n_chunks - 1) commit(mb_accf(b));
