@@ -229,282 +229,7 @@ __global__ void __launch_bounds__(NTH, 1) moff_dftgemm_kernel(const FwdArgs a, c
         return bound > 0.f ? max(-100, min(100, ex)) : 0;
     };
 
-    if (warp >= NXW && warp < NXW + NGW) {
-        // ------------------------------- gridding warps -------------------------------
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(kRegsOther));
-        const int gw = warp - NXW, gt = tid - 32 * NXW;   // among the gridding warps and threads
-        // ---- decode ----
-        // voltage row of item (cp, t); for XP, cp = 4 c + v runs over the virtual pols of channel
-        // c and the row is pol X of channel c (pol Y for v = 1), the Y row following it
-        auto vrow = [&](int cp, int t) -> const VT* {
-            if constexpr (XP) {
-                const int c = cp >> 2, p = (cp & 3) == 1 ? 1 : 0;
-                return V + ((long long)t * (a.n_cp >> 1) + 2 * c + p) * (long long)A;
-            } else {
-                return V + ((long long)t * a.n_cp + cp) * (long long)A;
-            }
-        };
-        // gains of an antenna for (channel, pol) cp; XP: virtual pol v = cp & 3: X, Y, X + Y, X + iY,
-        // gy = phi_v g_Y (phi_2 = 1, phi_3 = i)
-        auto gain_of = [&](int cp, int aa, float2& gx, float2& gy) {
-            if constexpr (XP) {
-                const int c = cp >> 2, v = cp & 3, p = v == 1 ? 1 : 0;
-                gx = a.gains ? __ldg(a.gains + (size_t)(2 * c + p) * A + aa) : make_float2(1.f, 0.f);
-                gy = a.gains ? __ldg(a.gains + (size_t)(2 * c + 1) * A + aa) : make_float2(1.f, 0.f);
-                if (v == 3) gy = make_float2(-gy.y, gy.x);
-            } else {
-                gx = a.gains ? __ldg(a.gains + (size_t)cp * A + aa) : make_float2(1.f, 0.f);
-            }
-        };
-        // Thread gt decodes image gt mod 2 of a pair, antennas gt / 2 + NGT / 2 i.
-        const int img_d = gt & 1, ant0 = gt >> 1;
-        constexpr int ASTEP = NGT / 2;
-        constexpr int VPT = 2;                          // antennas per thread loaded a pair ahead
-        int dcp = beg / T, dt = beg - dcp * T;          // (channel*pol, time) of the next pair's first image
-        int gcp = -1;                                   // (channel, pol) of the powers summed
-        int g0cp = -1;                                  // (channel, pol) of the gains held
-        float2 g0[VPT] = {}, gy0[VPT] = {};
-        auto next_image = [&](int& cp, int& t) {
-            if (++t == T) {
-                t = 0;
-                ++cp;
-            }
-        };
-        // raw voltages of the thread's first antennas for the next pair of images, loaded a pair ahead so that
-        // the decode does not wait on HBM; further antennas are loaded when decoded
-        VT raw[VPT] = {}, rawy[VPT] = {};
-        auto prefetch = [&](int left) {                 // images left from (dcp, dt) on
-            int cp = dcp, t = dt;
-            if (img_d) next_image(cp, t);
-            if (img_d < left) {
-                const VT* base = vrow(cp, t) + ant0;
-#pragma unroll
-                for (int i = 0; i < VPT; ++i) {
-                    if (ant0 + ASTEP * i < A) {
-                        raw[i] = __ldg(base + ASTEP * i);
-                        if constexpr (XP) {
-                            if ((cp & 3) >= 2) rawy[i] = __ldg(base + A + ASTEP * i);
-                        }
-                    }
-                }
-            }
-        };
-        auto add_power = [&](int cp, int aa, float v) {
-            if (a.power != nullptr && cp >= 0) atomicAdd(a.power + (size_t)cp * A + aa, (double)v);
-        };
-        // decode + gain of pair p into voltage buffer p mod nvb; the even thread of an antenna sums the
-        // power of both images (the same thread throughout, so no barrier separates the updates); the
-        // largest component magnitudes go to vmax[p mod 16] (positive float bits order like unsigned
-        // integers); then the next pair's voltages are prefetched
-        auto decode = [&](int p) {
-            float2* vb = reinterpret_cast<float2*>(sVB + (nvb == 2 && (p & 1) ? (size_t)A * VBYTES : 0));
-            int cp1 = dcp, t1 = dt;                        // the second image
-            next_image(cp1, t1);
-            const bool both = 2 * p + 1 < n, there = img_d == 0 || both;
-            const int cp = img_d ? cp1 : dcp, t = img_d ? t1 : dt;
-            if (there && cp != g0cp) {
-#pragma unroll
-                for (int i = 0; i < VPT; ++i)
-                    if (ant0 + ASTEP * i < A) gain_of(cp, ant0 + ASTEP * i, g0[i], gy0[i]);
-                g0cp = cp;
-            }
-            const bool two = XP && (cp & 3) >= 2;          // virtual pol combining X and Y
-            float m = 0.f;
-            auto one = [&](int aa, VT r, VT ry, float2 gx, float2 gy) {
-                float2 vp = make_float2(0.f, 0.f);
-                if (there) {
-                    vp = cmul(gx, Volt<VDT>::dec(r));
-                    if constexpr (XP) {
-                        if (two) {
-                            const float2 w = cmul(gy, Volt<VDT>::dec(ry));
-                            vp.x += w.x;
-                            vp.y += w.y;
-                        }
-                    }
-                }
-                if constexpr (LP) {
-                    const __half2 hv = __floats2half2_rn(vp.x, vp.y);
-                    reinterpret_cast<uint32_t*>(vb)[2 * aa + img_d] = *reinterpret_cast<const uint32_t*>(&hv);
-                } else {
-                    vb[2 * aa + img_d] = vp;
-                }
-                m = fmaxf(m, fmaxf(fabsf(vp.x), fabsf(vp.y)));
-                return cnorm(vp);
-            };
-            auto power = [&](int aa, float n0, float n1) {
-                float pw = PW[aa];
-                if (dcp != gcp) {
-                    add_power(gcp, aa, pw);
-                    pw = 0.f;
-                }
-                pw += n0;
-                if (both && cp1 != dcp) {
-                    add_power(dcp, aa, pw);
-                    pw = 0.f;
-                }
-                PW[aa] = pw + n1;
-            };
-            // the warp's lanes walk the antennas together (the even lane needs its neighbour's power)
-            auto both_images = [&](int aa, VT r, VT ry, float2 gx, float2 gy) {
-                const float nn = aa < A ? one(aa, r, ry, gx, gy) : 0.f;
-                const float n1 = __shfl_down_sync(0xffffffffu, nn, 1);
-                if (img_d == 0 && aa < A) power(aa, nn, n1);
-            };
-#pragma unroll
-            for (int i = 0; i < VPT; ++i)
-                if (16 * gw + ASTEP * i < A) both_images(ant0 + ASTEP * i, raw[i], rawy[i], g0[i], gy0[i]);
-#pragma unroll 1
-            for (int a0 = 16 * gw + ASTEP * VPT; a0 < A; a0 += ASTEP) {
-                const int aa = a0 + (lane >> 1);
-                float2 gx = make_float2(1.f, 0.f), gy = gx;
-                VT r{}, ry{};
-                if (there && aa < A) {
-                    const VT* base = vrow(cp, t);
-                    gain_of(cp, aa, gx, gy);
-                    r = __ldg(base + aa);
-                    if constexpr (XP) {
-                        if (two) ry = __ldg(base + A + aa);
-                    }
-                }
-                both_images(aa, r, ry, gx, gy);
-            }
-            if (16 * gw < A) {
-                const unsigned bits = __float_as_uint(m);
-                const unsigned m0 = __reduce_max_sync(0xffffffffu, img_d ? 0u : bits);
-                const unsigned m1 = __reduce_max_sync(0xffffffffu, img_d ? bits : 0u);
-                if (lane < 2) atomicMax(vmax + 2 * (p & 15) + lane, lane ? m1 : m0);
-            }
-            // pair p - 8's words: its F has long been taken (stage 1 of pair p - 3 is done, so every transform
-            // warp has split pair p - 4), and none decodes pair p + 8 before this warp has decoded pair p
-            if (gt < 2) vmax[2 * ((p + 8) & 15) + gt] = 0u;
-            gcp = both ? cp1 : dcp;
-            next_image(dcp, dt);
-            next_image(dcp, dt);
-            prefetch(n - 2 * (p + 1));
-        };
-        auto flush_power = [&]() {
-            if (img_d == 0)
-                for (int aa = ant0; aa < A; aa += ASTEP) add_power(gcp, aa, PW[aa]);
-        };
-
-        // ---- gridding ----
-        float down0 = 1.f, down1 = 1.f;                 // 2^-s of the pair being gridded
-        auto scales = [&](int p) {
-            down0 = __uint_as_float((unsigned)(127 - exponent(p, 0)) << 23);
-            down1 = __uint_as_float((unsigned)(127 - exponent(p, 1)) << 23);
-        };
-        // slot position jj of this warp, of pair p, into E buffer p mod 2
-        auto grid = [&](int p, int jj) {
-            const unsigned char* vb = sVB + (nvb == 2 && (p & 1) ? (size_t)A * VBYTES : 0);
-            __half* sEp = sE + (p & 1) * EBUF;
-            const int slot = PER_WARP * gw + jj;
-            const int2 sl = ldt<SMT>(tSlot + slot);              // first entry, steps (-1: no slot here)
-            if (sl.y < 0) return;
-            const uint32_t word = __ldg(g.lane + slot * 32 + lane);
-            __half* dst = sEp + (word & 0xffffu);
-            if (sl.y == 0) {                                     // no antenna reaches these cells
-#pragma unroll
-                for (int i = 0; i < (LP ? 4 : 8); ++i)
-                    *reinterpret_cast<uint32_t*>(dst + (i & 1) * EIMG + ((i >> 1) & 1) * NG * NG + (i >> 2) * EPART) = 0u;
-                return;
-            }
-            const ulonglong2 rt = __ldg(reinterpret_cast<const ulonglong2*>(rot + (word >> 16)));
-            float r[2][2] = {}, im[2][2] = {};                   // [image][cell]
-            // two steps at a time: both steps' table loads, then their voltage loads, so that two
-            // dependent load chains overlap
-            auto steps = [&](auto cw_tag, auto n_tag, int e) {   // cw_tag: complex weights (tWim) or not
-                constexpr bool CW = decltype(cw_tag)::value;
-                constexpr int U = decltype(n_tag)::value;
-                float2 w[U], wi[U];
-                float4 v[U];
-                int an[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    w[u] = ldt<SMT>(tWre + e + 32 * u);
-                    if constexpr (CW) wi[u] = ldt<SMT>(tWim + e + 32 * u);
-                    an[u] = ldt<SMT>(tAnt + e + 32 * u);
-                }
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    if constexpr (LP) {
-                        const uint2 q = reinterpret_cast<const uint2*>(vb)[an[u]];
-                        const float2 va = __half22float2(*reinterpret_cast<const __half2*>(&q.x));
-                        const float2 vc = __half22float2(*reinterpret_cast<const __half2*>(&q.y));
-                        v[u] = make_float4(va.x, va.y, vc.x, vc.y);
-                        // weights rounded to FP16, so that every product is exact in FP32
-                        w[u] = make_float2(round_h(w[u].x), round_h(w[u].y));
-                        if constexpr (CW) wi[u] = make_float2(round_h(wi[u].x), round_h(wi[u].y));
-                    } else {
-                        v[u] = reinterpret_cast<const float4*>(vb)[an[u]];
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < U; ++u)
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        const float wr = c ? w[u].y : w[u].x;
-                        r[0][c] = fmaf(wr, v[u].x, r[0][c]);
-                        im[0][c] = fmaf(wr, v[u].y, im[0][c]);
-                        r[1][c] = fmaf(wr, v[u].z, r[1][c]);
-                        im[1][c] = fmaf(wr, v[u].w, im[1][c]);
-                        if constexpr (CW) {
-                            const float wq = c ? wi[u].y : wi[u].x;
-                            r[0][c] = fmaf(-wq, v[u].y, r[0][c]);
-                            im[0][c] = fmaf(wq, v[u].x, im[0][c]);
-                            r[1][c] = fmaf(-wq, v[u].w, r[1][c]);
-                            im[1][c] = fmaf(wq, v[u].z, im[1][c]);
-                        }
-                    }
-            };
-            auto walk = [&](auto cw_tag) {
-                int e = sl.x + lane, k = sl.y;
-                for (; k >= 2; k -= 2, e += 64) steps(cw_tag, std::integral_constant<int, 2>{}, e);
-                if (k) steps(cw_tag, std::integral_constant<int, 1>{}, e);
-            };
-            if (tWim) walk(std::true_type{});
-            else walk(std::false_type{});
-            // rotate by exp(-i pi (x + y) / NP), scale, split and store y, y + 1 as one word
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const unsigned long long dn = f2dup(i ? down1 : down0);
-                const unsigned long long c = f2mul(rt.x, dn), s = f2mul(rt.y, dn);
-                const unsigned long long re = pack2(make_float2(r[i][0], r[i][1])), ii = pack2(make_float2(im[i][0], im[i][1]));
-                const unsigned long long ro = f2fma(re, c, f2mul(ii, s)), io = f2sub(f2mul(ii, c), f2mul(re, s));
-                __half* d = dst + i * EIMG;
-                if constexpr (LP) {
-                    *reinterpret_cast<uint32_t*>(d) = half_pair(ro);
-                    *reinterpret_cast<uint32_t*>(d + NG * NG) = half_pair(io);
-                } else {
-                    uint32_t rh, rl, ih, il;
-                    split2(ro, rh, rl);
-                    split2(io, ih, il);
-                    *reinterpret_cast<uint32_t*>(d) = rh;
-                    *reinterpret_cast<uint32_t*>(d + NG * NG) = ih;
-                    *reinterpret_cast<uint32_t*>(d + EPART) = rl;
-                    *reinterpret_cast<uint32_t*>(d + EPART + NG * NG) = il;
-                }
-            }
-        };
-        bool ok = true;
-        if (np > 0) prefetch(n);
-#pragma unroll 1
-        for (int p = 0; p < np; ++p) {
-            // with one voltage buffer, every warp's gridding of pair p - 1 comes first
-            if (nvb == 1 && p > 0 && !(ok = warp_wait(MB_EFULL + ((p - 1) & 1), (p - 1) >> 1))) break;
-            decode(p);
-            warp_arrive(MB_VFULL);
-            if (!(ok = warp_wait(MB_VFULL, p))) break;              // every warp has decoded the pair
-            scales(p);
-            // the E buffer is free once stage 1 of pair p - 2 has read it
-            if (p >= 2 && !(ok = warp_wait(MB_EFREE + (p & 1), (p - 2) >> 1))) break;
-#pragma unroll 1
-            for (int jj = 0; jj < PER_WARP; ++jj) grid(p, jj);
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // E^T visible to the tensor cores
-            warp_arrive(MB_EFULL + (p & 1));
-        }
-        if (ok && np > 0) flush_power();
-        if (!ok) *s_fail = 1;
-    } else if (warp < NXW) {
+    if (warp < NXW) {
         // ------------------------------- transform warps -------------------------------
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" :: "n"(kRegsTransform));
         const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
@@ -624,66 +349,344 @@ __global__ void __launch_bounds__(NTH, 1) moff_dftgemm_kernel(const FwdArgs a, c
         }
         if (!ok) *s_fail = 1;
     } else {
-        // ------------------------------- issuer -------------------------------
+        // the gridding warps and the issuer: one instruction for all of them, since the last warpgroup holds both and a
+        // warpgroup's four warps have to execute the same setmaxnreg
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(kRegsOther));
-        if (lane == 0 && np > 0) {
-        const uint64_t dW = sdesc(smem_u32(sW), 1024), dE = sdesc(smem_u32(sE), 1024);
-        constexpr int kWLo = 2 * WTAB / 16, kELo = 2 * EPART / 16, kEBuf = 2 * EBUF / 16, kEImg = 2 * EIMG / 16;
-        constexpr int NPROD = LP ? 1 : 3;               // hi hi, hi lo, lo hi (LP: hi hi only)
-        auto wait = [&](int i, int parity) { return mbar_wait(mb(i), (uint32_t)parity & 1u, a.wait_tries); };
-        auto stage2 = [&](int img) {
-            constexpr uint32_t id = idesc(128);
-            const uint32_t xa = tX + 128 * img;
-#pragma unroll
-            for (int q = 0; q < NPROD; ++q)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const uint32_t xop = xa + 16 * k + (q == 2 ? 64 : 0);
-                    const uint64_t b = dW + (uint64_t)((q == 1 ? kWLo : 0) + 16 * k);
-                    mma_ts(tF, xop, b, id, (q | k) != 0);
-                    mma_ts(tF + 128, xop + 8, b, id, (q | k) != 0);
+        if (warp < NXW + NGW) {
+            // ------------------------------- gridding warps -------------------------------
+            const int gw = warp - NXW, gt = tid - 32 * NXW;   // among the gridding warps and threads
+            // ---- decode ----
+            // voltage row of item (cp, t); for XP, cp = 4 c + v runs over the virtual pols of channel
+            // c and the row is pol X of channel c (pol Y for v = 1), the Y row following it
+            auto vrow = [&](int cp, int t) -> const VT* {
+                if constexpr (XP) {
+                    const int c = cp >> 2, p = (cp & 3) == 1 ? 1 : 0;
+                    return V + ((long long)t * (a.n_cp >> 1) + 2 * c + p) * (long long)A;
+                } else {
+                    return V + ((long long)t * a.n_cp + cp) * (long long)A;
                 }
-            commit(mb(MB_F));
-        };
-        bool ok = true, issued = false;
-        const int ni = 2 * np;
-        // stage 1 of image i, once its pair is gridded
-        auto stage1 = [&](int i) -> bool {
-            const int j = i >> 1, img = i & 1;
-            if (img == 0 && !wait(MB_EFULL + (j & 1), j >> 1)) return false;
-            fence_after();
-            constexpr uint32_t id1 = idesc(128);
-            const uint64_t e0 = dE + (uint64_t)((j & 1) * kEBuf + img * kEImg);
+            };
+            // gains of an antenna for (channel, pol) cp; XP: virtual pol v = cp & 3: X, Y, X + Y, X + iY,
+            // gy = phi_v g_Y (phi_2 = 1, phi_3 = i)
+            auto gain_of = [&](int cp, int aa, float2& gx, float2& gy) {
+                if constexpr (XP) {
+                    const int c = cp >> 2, v = cp & 3, p = v == 1 ? 1 : 0;
+                    gx = a.gains ? __ldg(a.gains + (size_t)(2 * c + p) * A + aa) : make_float2(1.f, 0.f);
+                    gy = a.gains ? __ldg(a.gains + (size_t)(2 * c + 1) * A + aa) : make_float2(1.f, 0.f);
+                    if (v == 3) gy = make_float2(-gy.y, gy.x);
+                } else {
+                    gx = a.gains ? __ldg(a.gains + (size_t)cp * A + aa) : make_float2(1.f, 0.f);
+                }
+            };
+            // Thread gt decodes image gt mod 2 of a pair, antennas gt / 2 + NGT / 2 i.
+            const int img_d = gt & 1, ant0 = gt >> 1;
+            constexpr int ASTEP = NGT / 2;
+            constexpr int VPT = 2;                          // antennas per thread loaded a pair ahead
+            int dcp = beg / T, dt = beg - dcp * T;          // (channel*pol, time) of the next pair's first image
+            int gcp = -1;                                   // (channel, pol) of the powers summed
+            int g0cp = -1;                                  // (channel, pol) of the gains held
+            float2 g0[VPT] = {}, gy0[VPT] = {};
+            auto next_image = [&](int& cp, int& t) {
+                if (++t == T) {
+                    t = 0;
+                    ++cp;
+                }
+            };
+            // raw voltages of the thread's first antennas for the next pair of images, loaded a pair ahead so that
+            // the decode does not wait on HBM; further antennas are loaded when decoded
+            VT raw[VPT] = {}, rawy[VPT] = {};
+            auto prefetch = [&](int left) {                 // images left from (dcp, dt) on
+                int cp = dcp, t = dt;
+                if (img_d) next_image(cp, t);
+                if (img_d < left) {
+                    const VT* base = vrow(cp, t) + ant0;
 #pragma unroll
-            for (int q = 0; q < NPROD; ++q)
+                    for (int i = 0; i < VPT; ++i) {
+                        if (ant0 + ASTEP * i < A) {
+                            raw[i] = __ldg(base + ASTEP * i);
+                            if constexpr (XP) {
+                                if ((cp & 3) >= 2) rawy[i] = __ldg(base + A + ASTEP * i);
+                            }
+                        }
+                    }
+                }
+            };
+            auto add_power = [&](int cp, int aa, float v) {
+                if (a.power != nullptr && cp >= 0) atomicAdd(a.power + (size_t)cp * A + aa, (double)v);
+            };
+            // decode + gain of pair p into voltage buffer p mod nvb; the even thread of an antenna sums the
+            // power of both images (the same thread throughout, so no barrier separates the updates); the
+            // largest component magnitudes go to vmax[p mod 16] (positive float bits order like unsigned
+            // integers); then the next pair's voltages are prefetched
+            auto decode = [&](int p) {
+                float2* vb = reinterpret_cast<float2*>(sVB + (nvb == 2 && (p & 1) ? (size_t)A * VBYTES : 0));
+                int cp1 = dcp, t1 = dt;                        // the second image
+                next_image(cp1, t1);
+                const bool both = 2 * p + 1 < n, there = img_d == 0 || both;
+                const int cp = img_d ? cp1 : dcp, t = img_d ? t1 : dt;
+                if (there && cp != g0cp) {
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    mma_ss(tX + 128 * img, dW + (uint64_t)((q == 2 ? kWLo : 0) + 16 * k),
-                           e0 + (uint64_t)((q == 1 ? kELo : 0) + 16 * k), id1, (q | k) != 0);
-            commit(mb(MB_ST1 + img));
-            if (img == 1) commit(mb(MB_EFREE + (j & 1)));
-            issued = true;
-            return true;
-        };
-        ok = stage1(0) && stage1(1);
+                    for (int i = 0; i < VPT; ++i)
+                        if (ant0 + ASTEP * i < A) gain_of(cp, ant0 + ASTEP * i, g0[i], gy0[i]);
+                    g0cp = cp;
+                }
+                const bool two = XP && (cp & 3) >= 2;          // virtual pol combining X and Y
+                float m = 0.f;
+                auto one = [&](int aa, VT r, VT ry, float2 gx, float2 gy) {
+                    float2 vp = make_float2(0.f, 0.f);
+                    if (there) {
+                        vp = cmul(gx, Volt<VDT>::dec(r));
+                        if constexpr (XP) {
+                            if (two) {
+                                const float2 w = cmul(gy, Volt<VDT>::dec(ry));
+                                vp.x += w.x;
+                                vp.y += w.y;
+                            }
+                        }
+                    }
+                    if constexpr (LP) {
+                        const __half2 hv = __floats2half2_rn(vp.x, vp.y);
+                        reinterpret_cast<uint32_t*>(vb)[2 * aa + img_d] = *reinterpret_cast<const uint32_t*>(&hv);
+                    } else {
+                        vb[2 * aa + img_d] = vp;
+                    }
+                    m = fmaxf(m, fmaxf(fabsf(vp.x), fabsf(vp.y)));
+                    return cnorm(vp);
+                };
+                auto power = [&](int aa, float n0, float n1) {
+                    float pw = PW[aa];
+                    if (dcp != gcp) {
+                        add_power(gcp, aa, pw);
+                        pw = 0.f;
+                    }
+                    pw += n0;
+                    if (both && cp1 != dcp) {
+                        add_power(dcp, aa, pw);
+                        pw = 0.f;
+                    }
+                    PW[aa] = pw + n1;
+                };
+                // the warp's lanes walk the antennas together (the even lane needs its neighbour's power)
+                auto both_images = [&](int aa, VT r, VT ry, float2 gx, float2 gy) {
+                    const float nn = aa < A ? one(aa, r, ry, gx, gy) : 0.f;
+                    const float n1 = __shfl_down_sync(0xffffffffu, nn, 1);
+                    if (img_d == 0 && aa < A) power(aa, nn, n1);
+                };
+#pragma unroll
+                for (int i = 0; i < VPT; ++i)
+                    if (16 * gw + ASTEP * i < A) both_images(ant0 + ASTEP * i, raw[i], rawy[i], g0[i], gy0[i]);
 #pragma unroll 1
-        for (int i = 0; ok && i < ni; ++i) {
-            const int j = i >> 1, img = i & 1;
-            if (!(ok = wait(MB_XA + img, j))) break;
-            if (i > 0 && !(ok = wait(MB_FREE, i - 1))) break;
-            fence_after();
-            stage2(img);
-            if (i + 2 < ni) {
-                if (!(ok = wait(MB_F, i))) break;           // stage 2 has read the columns stage 1 overwrites
-                ok = stage1(i + 2);
+                for (int a0 = 16 * gw + ASTEP * VPT; a0 < A; a0 += ASTEP) {
+                    const int aa = a0 + (lane >> 1);
+                    float2 gx = make_float2(1.f, 0.f), gy = gx;
+                    VT r{}, ry{};
+                    if (there && aa < A) {
+                        const VT* base = vrow(cp, t);
+                        gain_of(cp, aa, gx, gy);
+                        r = __ldg(base + aa);
+                        if constexpr (XP) {
+                            if (two) ry = __ldg(base + A + aa);
+                        }
+                    }
+                    both_images(aa, r, ry, gx, gy);
+                }
+                if (16 * gw < A) {
+                    const unsigned bits = __float_as_uint(m);
+                    const unsigned m0 = __reduce_max_sync(0xffffffffu, img_d ? 0u : bits);
+                    const unsigned m1 = __reduce_max_sync(0xffffffffu, img_d ? bits : 0u);
+                    if (lane < 2) atomicMax(vmax + 2 * (p & 15) + lane, lane ? m1 : m0);
+                }
+                // pair p - 8's words: its F has long been taken (stage 1 of pair p - 3 is done, so every transform
+                // warp has split pair p - 4), and none decodes pair p + 8 before this warp has decoded pair p
+                if (gt < 2) vmax[2 * ((p + 8) & 15) + gt] = 0u;
+                gcp = both ? cp1 : dcp;
+                next_image(dcp, dt);
+                next_image(dcp, dt);
+                prefetch(n - 2 * (p + 1));
+            };
+            auto flush_power = [&]() {
+                if (img_d == 0)
+                    for (int aa = ant0; aa < A; aa += ASTEP) add_power(gcp, aa, PW[aa]);
+            };
+
+            // ---- gridding ----
+            float down0 = 1.f, down1 = 1.f;                 // 2^-s of the pair being gridded
+            auto scales = [&](int p) {
+                down0 = __uint_as_float((unsigned)(127 - exponent(p, 0)) << 23);
+                down1 = __uint_as_float((unsigned)(127 - exponent(p, 1)) << 23);
+            };
+            // slot position jj of this warp, of pair p, into E buffer p mod 2
+            auto grid = [&](int p, int jj) {
+                const unsigned char* vb = sVB + (nvb == 2 && (p & 1) ? (size_t)A * VBYTES : 0);
+                __half* sEp = sE + (p & 1) * EBUF;
+                const int slot = PER_WARP * gw + jj;
+                const int2 sl = ldt<SMT>(tSlot + slot);              // first entry, steps (-1: no slot here)
+                if (sl.y < 0) return;
+                const uint32_t word = __ldg(g.lane + slot * 32 + lane);
+                __half* dst = sEp + (word & 0xffffu);
+                if (sl.y == 0) {                                     // no antenna reaches these cells
+#pragma unroll
+                    for (int i = 0; i < (LP ? 4 : 8); ++i)
+                        *reinterpret_cast<uint32_t*>(dst + (i & 1) * EIMG + ((i >> 1) & 1) * NG * NG + (i >> 2) * EPART) = 0u;
+                    return;
+                }
+                const ulonglong2 rt = __ldg(reinterpret_cast<const ulonglong2*>(rot + (word >> 16)));
+                float r[2][2] = {}, im[2][2] = {};                   // [image][cell]
+                // two steps at a time: both steps' table loads, then their voltage loads, so that two
+                // dependent load chains overlap
+                auto steps = [&](auto cw_tag, auto n_tag, int e) {   // cw_tag: complex weights (tWim) or not
+                    constexpr bool CW = decltype(cw_tag)::value;
+                    constexpr int U = decltype(n_tag)::value;
+                    float2 w[U], wi[U];
+                    float4 v[U];
+                    int an[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        w[u] = ldt<SMT>(tWre + e + 32 * u);
+                        if constexpr (CW) wi[u] = ldt<SMT>(tWim + e + 32 * u);
+                        an[u] = ldt<SMT>(tAnt + e + 32 * u);
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        if constexpr (LP) {
+                            const uint2 q = reinterpret_cast<const uint2*>(vb)[an[u]];
+                            const float2 va = __half22float2(*reinterpret_cast<const __half2*>(&q.x));
+                            const float2 vc = __half22float2(*reinterpret_cast<const __half2*>(&q.y));
+                            v[u] = make_float4(va.x, va.y, vc.x, vc.y);
+                            // weights rounded to FP16, so that every product is exact in FP32
+                            w[u] = make_float2(round_h(w[u].x), round_h(w[u].y));
+                            if constexpr (CW) wi[u] = make_float2(round_h(wi[u].x), round_h(wi[u].y));
+                        } else {
+                            v[u] = reinterpret_cast<const float4*>(vb)[an[u]];
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            const float wr = c ? w[u].y : w[u].x;
+                            r[0][c] = fmaf(wr, v[u].x, r[0][c]);
+                            im[0][c] = fmaf(wr, v[u].y, im[0][c]);
+                            r[1][c] = fmaf(wr, v[u].z, r[1][c]);
+                            im[1][c] = fmaf(wr, v[u].w, im[1][c]);
+                            if constexpr (CW) {
+                                const float wq = c ? wi[u].y : wi[u].x;
+                                r[0][c] = fmaf(-wq, v[u].y, r[0][c]);
+                                im[0][c] = fmaf(wq, v[u].x, im[0][c]);
+                                r[1][c] = fmaf(-wq, v[u].w, r[1][c]);
+                                im[1][c] = fmaf(wq, v[u].z, im[1][c]);
+                            }
+                        }
+                };
+                auto walk = [&](auto cw_tag) {
+                    int e = sl.x + lane, k = sl.y;
+                    for (; k >= 2; k -= 2, e += 64) steps(cw_tag, std::integral_constant<int, 2>{}, e);
+                    if (k) steps(cw_tag, std::integral_constant<int, 1>{}, e);
+                };
+                if (tWim) walk(std::true_type{});
+                else walk(std::false_type{});
+                // rotate by exp(-i pi (x + y) / NP), scale, split and store y, y + 1 as one word
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const unsigned long long dn = f2dup(i ? down1 : down0);
+                    const unsigned long long c = f2mul(rt.x, dn), s = f2mul(rt.y, dn);
+                    const unsigned long long re = pack2(make_float2(r[i][0], r[i][1])), ii = pack2(make_float2(im[i][0], im[i][1]));
+                    const unsigned long long ro = f2fma(re, c, f2mul(ii, s)), io = f2sub(f2mul(ii, c), f2mul(re, s));
+                    __half* d = dst + i * EIMG;
+                    if constexpr (LP) {
+                        *reinterpret_cast<uint32_t*>(d) = half_pair(ro);
+                        *reinterpret_cast<uint32_t*>(d + NG * NG) = half_pair(io);
+                    } else {
+                        uint32_t rh, rl, ih, il;
+                        split2(ro, rh, rl);
+                        split2(io, ih, il);
+                        *reinterpret_cast<uint32_t*>(d) = rh;
+                        *reinterpret_cast<uint32_t*>(d + NG * NG) = ih;
+                        *reinterpret_cast<uint32_t*>(d + EPART) = rl;
+                        *reinterpret_cast<uint32_t*>(d + EPART + NG * NG) = il;
+                    }
+                }
+            };
+            bool ok = true;
+            if (np > 0) prefetch(n);
+#pragma unroll 1
+            for (int p = 0; p < np; ++p) {
+                // with one voltage buffer, every warp's gridding of pair p - 1 comes first
+                if (nvb == 1 && p > 0 && !(ok = warp_wait(MB_EFULL + ((p - 1) & 1), (p - 1) >> 1))) break;
+                decode(p);
+                warp_arrive(MB_VFULL);
+                if (!(ok = warp_wait(MB_VFULL, p))) break;              // every warp has decoded the pair
+                scales(p);
+                // the E buffer is free once stage 1 of pair p - 2 has read it
+                if (p >= 2 && !(ok = warp_wait(MB_EFREE + (p & 1), (p - 2) >> 1))) break;
+#pragma unroll 1
+                for (int jj = 0; jj < PER_WARP; ++jj) grid(p, jj);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // E^T visible to the tensor cores
+                warp_arrive(MB_EFULL + (p & 1));
             }
-        }
-        // every MMA issued has completed before the tensor memory is released (full limit)
-        if (issued) {
-            commit(mb(MB_DRAIN));
-            mbar_wait(mb(MB_DRAIN), 0);
-        }
-        if (!ok) *s_fail = 1;
+            if (ok && np > 0) flush_power();
+            if (!ok) *s_fail = 1;
+        } else {
+            // ------------------------------- issuer -------------------------------
+            if (lane == 0 && np > 0) {
+            const uint64_t dW = sdesc(smem_u32(sW), 1024), dE = sdesc(smem_u32(sE), 1024);
+            constexpr int kWLo = 2 * WTAB / 16, kELo = 2 * EPART / 16, kEBuf = 2 * EBUF / 16, kEImg = 2 * EIMG / 16;
+            constexpr int NPROD = LP ? 1 : 3;               // hi hi, hi lo, lo hi (LP: hi hi only)
+            auto wait = [&](int i, int parity) { return mbar_wait(mb(i), (uint32_t)parity & 1u, a.wait_tries); };
+            auto stage2 = [&](int img) {
+                constexpr uint32_t id = idesc(128);
+                const uint32_t xa = tX + 128 * img;
+#pragma unroll
+                for (int q = 0; q < NPROD; ++q)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const uint32_t xop = xa + 16 * k + (q == 2 ? 64 : 0);
+                        const uint64_t b = dW + (uint64_t)((q == 1 ? kWLo : 0) + 16 * k);
+                        mma_ts(tF, xop, b, id, (q | k) != 0);
+                        mma_ts(tF + 128, xop + 8, b, id, (q | k) != 0);
+                    }
+                commit(mb(MB_F));
+            };
+            bool ok = true, issued = false;
+            const int ni = 2 * np;
+            // stage 1 of image i, once its pair is gridded
+            auto stage1 = [&](int i) -> bool {
+                const int j = i >> 1, img = i & 1;
+                if (img == 0 && !wait(MB_EFULL + (j & 1), j >> 1)) return false;
+                fence_after();
+                constexpr uint32_t id1 = idesc(128);
+                const uint64_t e0 = dE + (uint64_t)((j & 1) * kEBuf + img * kEImg);
+#pragma unroll
+                for (int q = 0; q < NPROD; ++q)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        mma_ss(tX + 128 * img, dW + (uint64_t)((q == 2 ? kWLo : 0) + 16 * k),
+                               e0 + (uint64_t)((q == 1 ? kELo : 0) + 16 * k), id1, (q | k) != 0);
+                commit(mb(MB_ST1 + img));
+                if (img == 1) commit(mb(MB_EFREE + (j & 1)));
+                issued = true;
+                return true;
+            };
+            ok = stage1(0) && stage1(1);
+#pragma unroll 1
+            for (int i = 0; ok && i < ni; ++i) {
+                const int j = i >> 1, img = i & 1;
+                if (!(ok = wait(MB_XA + img, j))) break;
+                if (i > 0 && !(ok = wait(MB_FREE, i - 1))) break;
+                fence_after();
+                stage2(img);
+                if (i + 2 < ni) {
+                    if (!(ok = wait(MB_F, i))) break;           // stage 2 has read the columns stage 1 overwrites
+                    ok = stage1(i + 2);
+                }
+            }
+            // every MMA issued has completed before the tensor memory is released (full limit)
+            if (issued) {
+                commit(mb(MB_DRAIN));
+                mbar_wait(mb(MB_DRAIN), 0);
+            }
+            if (!ok) *s_fail = 1;
+            }
         }
     }
 
