@@ -88,10 +88,11 @@ cudaError_t launch_finalize_xpol(const double* accum4, float* image, float2* cro
 constexpr int kAcThreads = 512;
 constexpr int kAcMaxCluster = 8;
 
-// A cluster of n_cl CTAs per (channel, pol).  Shared: U [L*L] float2, the CTA's part of U [L*L] float2,
-// T1 [L][N_p] float2, twiddles [N_p] float2, the CTA's share of the powers.  Phases:
+// A cluster of n_cl CTAs per (channel, pol).  Shared: U [L*L] float2, T1 [L][N_p] float2, twiddles [N_p] float2,
+// the CTA's share of the powers.  Phases:
 //   U(d)        = sum_a P_a R_a(d)                       (L^2 x A multiply-adds): each CTA sums its share of
-//                 the antennas, kAcThreads / L^2 of them side by side, then every CTA adds up the parts
+//                 the antennas, kAcThreads / L^2 of them side by side, into T1's space (L <= N_p - 1), then every
+//                 CTA adds up the parts
 //   T1(dy, kx)  = sum_dx U(dy, dx) exp(+2 pi i dx kx / N_p) (L^2 x N_p, in every CTA)
 //   A(ky, kx)   = Re sum_dy T1(dy, kx) exp(+2 pi i dy ky / N_p)  (N_p^2 x L, split over the CTAs)
 // with k measured from the image centre (k = pixel - N_p/2; the exponent is periodic).  With an image
@@ -108,8 +109,7 @@ autocorr_kernel(const double* __restrict__ power, const float2* __restrict__ lag
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int LL = L * L, h = (L - 1) / 2, msk = n_pad - 1;
     float2* U = reinterpret_cast<float2*>(smem_raw);
-    float2* UP = U + LL;
-    float2* T1 = UP + LL;
+    float2* T1 = U + LL;
     float2* TWs = T1 + L * n_pad;
     const int n_cl = (int)cg::this_cluster().num_blocks(), rank = (int)cg::this_cluster().block_rank();
     const int cp = blockIdx.x / n_cl;
@@ -137,15 +137,15 @@ autocorr_kernel(const double* __restrict__ power, const float2* __restrict__ lag
     for (int j = threadIdx.x; j < LL; j += blockDim.x) {
         float2 u = T1[j];
         for (int g = 1; g < G; ++g) u = cadd(u, T1[g * LL + j]);
-        UP[j] = u;
+        T1[j] = u;                   // read by this thread alone until the clusters meet
     }
     cg::this_cluster().sync();
     for (int j = threadIdx.x; j < LL; j += blockDim.x) {
         float2 u = make_float2(0.f, 0.f);
-        for (int r = 0; r < n_cl; ++r) u = cadd(u, *cluster_ptr(UP + j, r));
+        for (int r = 0; r < n_cl; ++r) u = cadd(u, *cluster_ptr(T1 + j, r));
         U[j] = u;
     }
-    cg::this_cluster().sync();       // the parts have been read: a CTA may leave; U is complete
+    cg::this_cluster().sync();       // the parts have been read: T1 may be written, a CTA may leave; U is complete
     for (int j = threadIdx.x; j < L * n_pad; j += blockDim.x) {
         const int dy = j / n_pad, ix = j % n_pad, kx = ix - n_pad / 2;
         float2 acc = make_float2(0.f, 0.f);
@@ -284,7 +284,7 @@ cudaError_t launch_isotropic(const float* image, const float* autocorr, const fl
     return cudaGetLastError();
 }
 
-// The size that decides whether a plan has the auto-correlation tables.
+// Shared memory of the kernel with all the powers in one CTA: decides whether a plan has the auto-correlation tables.
 size_t autocorr_smem_bytes(int lag_side, int n_pad, int n_ant) {
     return sizeof(float2) * ((size_t)lag_side * lag_side + (size_t)lag_side * n_pad + n_pad)
          + sizeof(float) * (size_t)n_ant;
@@ -297,19 +297,8 @@ cudaError_t launch_autocorr(const double* power, const float2* lag_tab, const fl
     while (n_cl < kAcMaxCluster && (long long)n_cp * n_cl < 2LL * n_sm && n_cl * 2 * 2 <= n_ant &&
            n_pad * n_pad >= kAcThreads * n_cl * 2)
         n_cl *= 2;
-    // a plan at the limit of autocorr_smem_bytes may leave no room for the second L^2 table with all its powers
-    auto need = [&](int k) {
-        return sizeof(float2) * (2 * (size_t)lag_side * lag_side + (size_t)lag_side * n_pad + n_pad)
-             + sizeof(float) * (size_t)((n_ant + k - 1) / k);
-    };
-    if (need(n_cl) > 48 * 1024) {
-        int dev = 0, optin = 0;
-        cudaError_t q = cudaGetDevice(&dev);
-        if (q == cudaSuccess) q = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        if (q != cudaSuccess) return q;
-        while (n_cl < kAcMaxCluster && need(n_cl) > (size_t)optin) n_cl *= 2;
-    }
-    const size_t smem = need(n_cl);
+    // at most autocorr_smem_bytes, which admitted the plan: the CTAs share out the powers
+    const size_t smem = autocorr_smem_bytes(lag_side, n_pad, (n_ant + n_cl - 1) / n_cl);
     cudaError_t e = ensure_smem<autocorr_kernel>(smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
