@@ -22,6 +22,7 @@ struct HalfGather {
     const int* ant_ptr = nullptr;
     const int2* ant_ent = nullptr;
     const float* ant_wim = nullptr;
+    int n_ent = 0;                  // entries of the mapping
 };
 
 // Everything a launch needs, all device pointers.

@@ -45,7 +45,7 @@ struct epic_plan {
     int2* hg_ant_ent = nullptr;
     float* hg_ant_wim = nullptr;
     epic::HalfGather half_gather() const {
-        return epic::HalfGather{hg_run, hg_w, hg_wim, hg_key, hg_empty, hg_ant_ptr, hg_ant_ent, hg_ant_wim};
+        return epic::HalfGather{hg_run, hg_w, hg_wim, hg_key, hg_empty, hg_ant_ptr, hg_ant_ent, hg_ant_wim, (int)nnz};
     }
     int* ant_ptr = nullptr;
     int2* ant_ent = nullptr;

@@ -1,4 +1,5 @@
 // Instantiation of the forward and adjoint MOFF kernels for N_p = 256.
+#include "half_rule.h"
 #include "moff_fwd.cuh"
 #include "moff_bwd.cuh"
 
@@ -6,20 +7,18 @@ namespace epic {
 
 // Which form.  The half-image kernels (moff_half256.cu) need every plan of the launch to have their table (up to
 // 1,471 antennas); the 4-CTA clusters take more antennas, the cross-polarisation products, a batch's request for one
-// row-pass buffer, and calls of few images, where a cluster finishes an image sooner than two SMs their halves.
-// Measured: a half image takes an SM 14.5 us and an image a cluster 7.8 us (331 antennas, 7.05 against 6.05 ms for
-// 32,768 images); the adjoint 33 and 20 us (1,024 antennas).  So the line lies where the waves of half
-// images over the SMs take less time than the waves of images over n_sm / 4 clusters.
-static bool half_pays(long long n_items, int n_sm, int half_cost, int cluster_cost) {
-    const long long n_cl = n_sm / 4 > 0 ? n_sm / 4 : 1;
-    return (2 * n_items + n_sm - 1) / n_sm * half_cost <= (n_items + n_cl - 1) / n_cl * cluster_cost;
-}
-
+// row-pass buffer, and the calls for which they are the faster form (half_rule.h).
 static bool use_half(const SegList& L, bool xpol, int n_sm) {
-    if (xpol || L.max_buffers == 1 || L.first[L.n_seg] >= 1 << 30) return false;   // half images in 32 bits
-    for (int s = 0; s < L.n_seg; ++s)
+    const long long n_items = L.first[L.n_seg];
+    if (xpol || L.max_buffers == 1 || n_items < 1 || n_items >= 1 << 30) return false;   // half images in 32 bits
+    double n_ent = 0.0;
+    long long n_cp = 0;
+    for (int s = 0; s < L.n_seg; ++s) {
         if (!L.seg[s].half.run) return false;
-    return half_pays(L.first[L.n_seg], n_sm, 15, 8);
+        n_ent += double(L.seg[s].half.n_ent) * double(L.first[s + 1] - L.first[s]) / double(n_items);
+        n_cp += L.seg[s].n_cp;
+    }
+    return half_pays_fwd(n_items, n_sm, n_ent, n_cp);
 }
 
 cudaError_t launch_fwd_256(int vdt, const SegList& L, int n_sm, cudaStream_t st, bool xpol) {
@@ -33,7 +32,7 @@ cudaError_t launch_fwd_256(int vdt, const SegList& L, int n_sm, cudaStream_t st,
 }
 
 cudaError_t launch_bwd_256(int vdt, const BwdArgs& a, int n_sm, cudaStream_t st) {
-    if (a.half.run && half_pays(a.n_items, n_sm, 33, 20)) return launch_half256_bwd(vdt, a, n_sm, st);
+    if (a.half.run && half_pays_bwd(a.n_items, n_sm, a.half.n_ent)) return launch_half256_bwd(vdt, a, n_sm, st);
     switch (vdt) {
         case 0: return launch_bwd_t<256, 0>(a, n_sm, st);
         case 1: return launch_bwd_t<256, 1>(a, n_sm, st);
