@@ -15,11 +15,12 @@
 
 namespace {
 
-// Kernel forms a size class can run in: the persistent one-launch form (one CTA, or one cluster
-// for N_p >= 256, per image in flight; at N_p = 256 with two row-pass buffers where they fit),
+// Kernel forms a size class can run in: the persistent one-launch form (one CTA per image in flight, one
+// cluster at N_p = 512; at N_p = 256 half images, or clusters with two row-pass buffers where
+// they fit: see launch_fwd_256),
 // for N_p = 512 the two-pass form (a row pass and a column pass over every SM, the row-
 // transformed grids staged in the class's scratch buffer), and for N_p = 256 the persistent form
-// with one row-pass buffer (less shared memory, a cluster barrier per item).
+// in clusters with one row-pass buffer (less shared memory, a cluster barrier per item).
 enum ClassForm { kFormPersistent = 0, kFormTwoPass = 1, kFormOneBuffer = 2 };
 
 struct ClassRun {
@@ -27,7 +28,7 @@ struct ClassRun {
     std::vector<int> members;      // plan indices (at most epic::kMaxSeg)
     cudaStream_t stream = nullptr;
     cudaEvent_t join = nullptr;
-    int max_workers = 0;           // 0 = every resident CTA (cluster)
+    int max_workers = 0;           // cap in CTAs (clusters; SMs at N_p = 256), 0 = every resident one
     int form = kFormPersistent;
     float2* scratch = nullptr;     // N_p = 512: the two-pass form's scratch (tp_chunk items)
     int tp_chunk = 0;
@@ -271,8 +272,8 @@ epic_status epic_batch_autotune(epic_batch* batch, const void* const* volt, cons
         return EPIC_OK;
     };
     // 1) per class: the kernel form and worker count that run it fastest alone -- the persistent
-    //    form with all, 3/4 or 1/2 of its resident CTAs (clusters), for N_p = 512 also the
-    //    two-pass form on every SM, for N_p = 256 also the one-buffer form at the best count
+    //    form with all, 3/4 or 1/2 of its resident CTAs (clusters; SMs at N_p = 256), for N_p = 512 also
+    //    the two-pass form on every SM, for N_p = 256 also the one-buffer form at the best count
     std::vector<float> alone(batch->classes.size(), 0.f);
     for (size_t k = 0; k < batch->classes.size() && s == EPIC_OK; ++k) {
         ClassRun& c = batch->classes[k];

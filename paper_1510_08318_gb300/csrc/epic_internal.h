@@ -69,9 +69,10 @@ struct SegList {
     long long cost[kMaxSeg + 1];  // cumulative cost before each sub-array; cost[n_seg] = total
     int n_seg;
     int max_ant;               // largest antenna count (shared-memory sizing)
-    int max_workers;           // cap on CTAs (clusters) launched, 0 = every resident one
-    int max_buffers = 0;       // FFT form's row-pass buffers: 1 = one, 0 = as many as fit (two at
-                               // N_p = 256)
+    int max_workers;           // cap on CTAs (clusters) launched, 0 = every resident one; in SMs at
+                               // N_p = 256 where every plan has its half images (half_rule.h)
+    int max_buffers = 0;       // 1: clusters with one row-pass buffer (N_p = 256), 0: the faster form,
+                               // with as many as fit
 };
 
 // Per-item cost estimate of a sub-array (relative units): transform work per padded pixel
@@ -177,7 +178,8 @@ int half256_row_stride();
 cudaError_t launch_half256_fwd(int vdt, const SegList& L, int n_sm, cudaStream_t st);
 cudaError_t launch_half256_bwd(int vdt, const BwdArgs& a, int n_sm, cudaStream_t st);
 
-// CTAs (Q = 1) or clusters (Q > 1) of the forward kernel resident on the whole GPU.
+// CTAs (Q = 1) or clusters (Q > 1) of the forward kernel resident on the whole GPU (N_p = 256: SMs where the
+// antennas fit the half images).
 int resident_fwd_workers(int n_pad, int vdt, int max_ant, int n_sm);
 template <int NP, int VDT> int resident_fwd_workers_t(int max_ant, int n_sm);
 

@@ -31,4 +31,17 @@ inline bool half_pays_bwd(long long n_items, int n_sm, double n_ent) {
     return half_waves(n_items, n_sm) * (23.0 + 8e-4 * n_ent) <= cluster_waves(n_items, n_sm) * (15.0 + 4e-4 * n_ent);
 }
 
+// The form of a forward launch whose plans all have their half images, and the cap on its CTAs or clusters (0: none).
+// A launch is capped in SMs (max_workers, 0: none), since the caller does not know the form: a cluster stands for four.
+struct HalfChoice {
+    bool half;
+    int cap;
+};
+inline HalfChoice half_choice(long long n_items, int n_sm, double n_ent, long long n_cp, int max_workers, bool one_buffer) {
+    const int sms = max_workers > 0 && max_workers < n_sm ? max_workers : n_sm;
+    // half images are numbered in 32 bits
+    if (!one_buffer && n_items < 1 << 30 && half_pays_fwd(n_items, sms, n_ent, n_cp)) return {true, max_workers};
+    return {false, max_workers > 0 ? (sms / 4 > 0 ? sms / 4 : 1) : 0};
+}
+
 }  // namespace epic

@@ -30,19 +30,23 @@ MEASURED = {
 CLEAR = 0.8
 
 
-@pytest.fixture(scope="module")
-def rule(tmp_path_factory):
+def _compiled(tmp_path_factory, body):
     cxx = shutil.which("g++") or shutil.which("c++")
     if cxx is None:
         pytest.skip("no C++ compiler")
     d = tmp_path_factory.mktemp("rule")
     src, exe = str(d / "rule.cpp"), str(d / "rule")
     with open(src, "w") as f:
-        f.write('#include "half_rule.h"\n#include <cstdio>\nint main() {\n    long long e, n, c;\n'
-                '    while (std::scanf("%lld %lld %lld", &e, &n, &c) == 3)\n'
-                '        std::printf("%d %d\\n", epic::half_pays_fwd(n, 152, double(e), c), '
-                'epic::half_pays_bwd(n, 152, double(e)));\n}\n')
+        f.write('#include "half_rule.h"\n#include <cstdio>\nint main() {\n    long long e, n, c, m, o;\n%s}\n' % body)
     subprocess.run([cxx, "-std=c++17", "-I" + CSRC, "-o", exe, src], check=True)
+    return exe
+
+
+@pytest.fixture(scope="module")
+def rule(tmp_path_factory):
+    exe = _compiled(tmp_path_factory, '    while (std::scanf("%lld %lld %lld", &e, &n, &c) == 3)\n'
+                    '        std::printf("%d %d\\n", epic::half_pays_fwd(n, 152, double(e), c), '
+                    'epic::half_pays_bwd(n, 152, double(e)));\n')
     text = "".join("%d %d %d\n" % (e, t * c, c) for e, t, c in MEASURED)
     out = subprocess.run([exe], input=text, capture_output=True, text=True, check=True).stdout.split()
     return {k: (out[2 * i] == "1", out[2 * i + 1] == "1") for i, k in enumerate(MEASURED)}
@@ -54,3 +58,26 @@ def test_choice(rule, case):
         assert (h if half else c) <= 1.05 * c
         if h < CLEAR * c and case[1] * case[2] > 38:
             assert half
+
+
+@pytest.mark.parametrize("items, n_ent, n_cp, cap, one_buffer, want", [
+    (4096, 3000, 32, 0, 0, (1, 0)),          # no cap
+    (4096, 3000, 32, 76, 0, (1, 76)),        # half images on 76 SMs
+    (4096, 3000, 32, 76, 1, (0, 19)),        # the same SMs as clusters of four
+    (4096, 3000, 32, 114, 1, (0, 28)),
+    (30, 3000, 1, 114, 0, (0, 28)),          # few images: clusters
+    (30, 3000, 1, 3, 0, (0, 1)),
+    (30, 3000, 1, 0, 0, (0, 0)),
+    (76, 3000, 4, 0, 0, (1, 0)),             # one wave of halves on 152 SMs, two on 76
+    (76, 3000, 4, 76, 0, (1, 76)),
+    (77, 3000, 4, 76, 0, (0, 19)),           # three waves of halves and five of clusters
+    (1 << 30, 3000, 32, 0, 0, (0, 0)),       # too many half images to number
+])
+def test_cap_in_sms(tmp_path_factory, items, n_ent, n_cp, cap, one_buffer, want):
+    """A launch is capped in SMs, whichever form it takes, and the rule counts the SMs under the cap."""
+    exe = _compiled(tmp_path_factory, '    std::scanf("%lld %lld %lld %lld %lld", &n, &e, &c, &m, &o);\n'
+                    '    const epic::HalfChoice f = epic::half_choice(n, 152, double(e), c, int(m), o != 0);\n'
+                    '    std::printf("%d %d\\n", f.half, f.cap);\n')
+    out = subprocess.run([exe], input="%d %d %d %d %d" % (items, n_ent, n_cp, cap, one_buffer), capture_output=True,
+                         text=True, check=True).stdout.split()
+    assert tuple(map(int, out)) == want
