@@ -18,7 +18,7 @@
 // where voltages are read one by one: two MMAs of N = 128, one with its A operand negated, for the second):
 // Re V in columns 0..127 and -Im V in 128..255.  The CTA's warps have three roles, handing work
 // over through mbarriers only (no CTA-wide barrier inside the loop):
-//   - sets of 8 decode warps (two, or three for voltages read one by one) take the chunks in turn and
+//   - sets of 8 decode warps (two, or three for long integrations read one by one) take the chunks in turn and
 //     convert their voltages (loaded into registers three of the set's chunks ahead) into one
 //     stage of a 3-stage ring; each warp fences
 //     its stores for the tensor cores and arrives on the stage's full barrier, and refills a
@@ -51,6 +51,7 @@
 #include <algorithm>
 #include <cuda_fp16.h>
 #include <cstdint>
+#include "launch_rules.h"
 #include "moff_common.cuh"
 #include "tcgen05.cuh"
 
@@ -71,12 +72,13 @@ constexpr int kRowStride = 18;
 // The roles of a CTA's warps (one CTA per SM).  Measured (us, 256 antennas, 256 (channel, pol), 4+4-bit voltages of
 // 1,024 and of 64 samples; sets, epilogue warps, stages): 2, 8, 3: 116 and 44; 3, 4, 3: 113 and 61; 2, 8, 4: 121 and
 // 45; 3, 4, 5: 119 and 61; 1, 8, 4: 193 and 54.  More stages leave less L1 for the loads in flight: FP16 voltages of
-// 1,024 samples (read one by one, so with three sets) take 192 with 3 stages and 257 with 5.
-template <bool WIDE>
+// 1,024 samples (read one by one, with three sets) take 192 with 3 stages and 257 with 5.  SHORT: the roles of a
+// short integration of voltages read one by one (xeng_short).
+template <bool WIDE, bool SHORT>
 struct Roles {
-    static constexpr int NDS = WIDE ? 2 : 3;                // decode warp sets, taking alternate chunks
+    static constexpr int NDS = WIDE || SHORT ? 2 : 3;       // decode warp sets, taking alternate chunks
     static constexpr int NDW = 8 * NDS;                     // decode warps (a set's tile mappings take 256 threads)
-    static constexpr int NEW = WIDE ? 8 : 4;                // epilogue warps, NEW / 4 per TMEM lane quarter
+    static constexpr int NEW = WIDE || SHORT ? 8 : 4;       // epilogue warps, NEW / 4 per TMEM lane quarter
     static constexpr int MMA_WARP = NDW;                    // the warp whose first thread issues the MMAs
     static constexpr int NT = 32 * (NDW + 1 + NEW);
     // the B tile with the plane -Re_b, or without: then its product is one MMA of N = 128 more with the A operand
@@ -128,9 +130,9 @@ __device__ __forceinline__ void unit_coords(int u, int nab, int& cp, int& ab, in
     bb = ab + r;
 }
 
-template <int VDT, bool WIDE>
-__global__ void __launch_bounds__(Roles<WIDE>::NT, 1) xeng_kernel(const XengArgs a) {
-    using W = Roles<WIDE>;
+template <int VDT, bool WIDE, bool SHORT>
+__global__ void __launch_bounds__(Roles<WIDE, SHORT>::NT, 1) xeng_kernel(const XengArgs a) {
+    using W = Roles<WIDE, SHORT>;
     constexpr int NDS = W::NDS, NDW = W::NDW, NEW = W::NEW, MMA_WARP = W::MMA_WARP, NSTAGE = W::NSTAGE, N_MBAR = W::N_MBAR;
     constexpr int kBTileBytes = W::kBTileBytes, kStageBytes = W::kStageBytes;
     static_assert(!WIDE || VDT == 2, "the wide loads are for 4+4-bit voltages");
@@ -437,9 +439,11 @@ __global__ void __launch_bounds__(Roles<WIDE>::NT, 1) xeng_kernel(const XengArgs
             float2* out = a.vis + (size_t)cp * A * A;
             // 16 columns at a time.  A lane holds a row, so the mirrored block is written 32 adjacent elements at a
             // time, and on the diagonal, where the block is its own mirror, it alone.  Off the diagonal the rows
-            // themselves go through shared memory, to be written 16 adjacent elements at a time.
+            // themselves go through shared memory, to be written 16 adjacent elements at a time.  Rows and columns past
+            // the last antenna are left out (130 antennas: the second block column holds two).
+            const int c1 = a0 + 32 * q < A ? min(c0 + 512 / NEW, A - b0) : c0;
 #pragma unroll 1
-            for (int c = c0; c < c0 + 512 / NEW; c += 16) {
+            for (int c = c0; c < c1; c += 16) {
 #pragma unroll
                 for (int h = 0; h < 16; h += 8) {
                     float dr[8], di[8];
@@ -815,7 +819,9 @@ cudaError_t launch_fx_image_t(const FxArgs& a, cudaStream_t st) {
 
 }  // namespace xe
 
-size_t xeng_smem_bytes() { return std::max(xe::Roles<false>::kSmem, xe::Roles<true>::kSmem); }
+size_t xeng_smem_bytes() {
+    return std::max({xe::Roles<false, false>::kSmem, xe::Roles<false, true>::kSmem, xe::Roles<true, false>::kSmem});
+}
 
 cudaError_t launch_fx_image(int n_pad, const FxArgs& a, cudaStream_t st) {
     if (a.n_cp == 0) return cudaSuccess;
@@ -828,13 +834,19 @@ cudaError_t launch_fx_image(int n_pad, const FxArgs& a, cudaStream_t st) {
 }
 
 namespace {
-template <int VDT, bool WIDE>
+template <int VDT, bool WIDE, bool SHORT>
 cudaError_t launch_xeng_t(const XengArgs& a, long long grid, cudaStream_t st) {
-    constexpr size_t smem = xe::Roles<WIDE>::kSmem;
-    const cudaError_t e = ensure_smem<xe::xeng_kernel<VDT, WIDE>>(smem);
+    constexpr size_t smem = xe::Roles<WIDE, SHORT>::kSmem;
+    const cudaError_t e = ensure_smem<xe::xeng_kernel<VDT, WIDE, SHORT>>(smem);
     if (e != cudaSuccess) return e;
-    xe::xeng_kernel<VDT, WIDE><<<(unsigned)grid, xe::Roles<WIDE>::NT, smem, st>>>(a);
+    xe::xeng_kernel<VDT, WIDE, SHORT><<<(unsigned)grid, xe::Roles<WIDE, SHORT>::NT, smem, st>>>(a);
     return cudaGetLastError();
+}
+
+template <int VDT>
+cudaError_t launch_xeng_singly(const XengArgs& a, long long grid, cudaStream_t st) {
+    return xeng_short(VDT == 1, a.n_time) ? launch_xeng_t<VDT, false, true>(a, grid, st)
+                                          : launch_xeng_t<VDT, false, false>(a, grid, st);
 }
 }  // namespace
 
@@ -846,12 +858,12 @@ cudaError_t launch_xeng(int vdt, const XengArgs& a, int n_sm, cudaStream_t st) {
     const long long grid = n_units < n_sm ? n_units : n_sm;
     switch (vdt) {
         case 1:
-            return launch_xeng_t<1, false>(a, grid, st);
+            return launch_xeng_singly<1>(a, grid, st);
         case 2:
             // 4-byte loads of 4 antennas need every group of 4 to start on a 4-byte boundary
             if (a.n_ant % 4 == 0 && reinterpret_cast<uintptr_t>(a.volt) % 4 == 0)
-                return launch_xeng_t<2, true>(a, grid, st);
-            return launch_xeng_t<2, false>(a, grid, st);
+                return launch_xeng_t<2, true, false>(a, grid, st);
+            return launch_xeng_singly<2>(a, grid, st);
         default:
             return cudaErrorInvalidValue;
     }
