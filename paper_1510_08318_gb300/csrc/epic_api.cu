@@ -1058,6 +1058,7 @@ epic_status epic_fx_image(const epic_plan* plan, const float* vis, float* image,
     a.n_ant = plan->n_ant;
     a.lag_ptr = plan->fx_lag_ptr;
     a.lag_ent = plan->fx_lag_ent;
+    a.n_ent = plan->fx_lag_n;
     a.vis_t = plan->fx_vis_t;
     a.u = plan->fx_u;
     a.image = image;

@@ -126,6 +126,7 @@ struct FxArgs {
     int n_cp, n_ant;
     const int* lag_ptr;        // [N_p^2 + 1] CSR of the antenna-pair kernels by wrapped lag cell
     const int4* lag_ent;       // {B_ab(d) re bits, im bits, pair * CP, 0} of each entry
+    long long n_ent;           // their number
     float2* vis_t;             // scratch [A (A + 1) / 2][CP]: the folded visibilities pair-major
     float2* u;                 // scratch [CP][N_p][N_p]: the lag planes
     float* image;              // [CP][N_p][N_p]

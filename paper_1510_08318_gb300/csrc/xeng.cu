@@ -590,7 +590,7 @@ __global__ void __launch_bounds__(256) fx_fold_kernel(const float2* __restrict__
 // with both orders of every pair gathered, G = 64 and 8-warp CTAs; 538 with one order; 412 with
 // G = 16 (a tile's pairs then mostly stay in L1); 286 with the tiles ordered by their distance from
 // lag 0; 229 with one 32-warp CTA per SM, which shortens the longest tiles fourfold (64 registers,
-// 4 loads in flight per lane).  The width G: see launch_fx_image_t.
+// 4 loads in flight per lane).  The width G: see fx_planes_per_group.
 constexpr int FXG_NT = 1024;
 
 template <int G, bool V4>
@@ -790,12 +790,7 @@ cudaError_t launch_fx_image_t(const FxArgs& a, cudaStream_t st) {
                           (unsigned)((a.n_cp + 31) / 32)), 256, 0, st>>>(a.vis, a.n_cp, a.n_ant, a.vis_t);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    // Planes per group: narrow groups keep more of a tile's pairs in L1 and give more CTAs, wide ones
-    // read each table entry and its row of visibilities fewer times.  Measured (us; 256 antennas,
-    // N_p = 128) with 2, 4, 8, 16, 32 planes per group: 4 planes 64, 68, 78, -, -; 8 planes 88, 72, 81,
-    // 107, -; 16 planes 167, 99, 89, 108, 171; 32 planes 310, 170, 107, 109, 181; 64 planes 616, 333,
-    // 198, 141, 189; 128 planes -, -, 367, 252, 229.
-    const int g = a.n_cp >= 96 ? 32 : a.n_cp >= 40 ? 16 : a.n_cp >= 12 ? 8 : a.n_cp >= 6 ? 4 : a.n_cp >= 2 ? 2 : 1;
+    const int g = fx_planes_per_group(a.n_cp, NP, a.n_ent);
     const unsigned blocks = (unsigned)((NP / 8) * (NP / 8) * (long long)((a.n_cp + g - 1) / g));
     switch (2 * g + (a.n_cp % 2 == 0 ? 1 : 0)) {
         case 2: fx_gather_kernel<1, false><<<blocks, FXG_NT, 0, st>>>(a, NP); break;
