@@ -10,6 +10,7 @@
 //                    A(k) = sum_d U(d) exp(+2 pi i d.k / N_p) with U(d) = sum_a P_a R_a(d):
 //                    a dense mat-vec over the small L x L lag window, then a separable sum
 //                    onto the N_p x N_p pixels (U is Hermitian, so A is real).
+#include "launch_rules.h"
 #include "moff_common.cuh"
 #include "moff_bwd.cuh"
 
@@ -86,7 +87,6 @@ cudaError_t launch_finalize_xpol(const double* accum4, float* image, float2* cro
 }
 
 constexpr int kAcThreads = 512;
-constexpr int kAcMaxCluster = 8;
 
 // A cluster of n_cl CTAs per (channel, pol).  Shared: U [L*L] float2, T1 [L][N_p] float2, twiddles [N_p] float2,
 // the CTA's share of the powers.  Phases:
@@ -292,11 +292,7 @@ size_t autocorr_smem_bytes(int lag_side, int n_pad, int n_ant) {
 
 cudaError_t launch_autocorr(const double* power, const float2* lag_tab, const float2* twiddle, int n_cp, int n_ant, int lag_side, int n_pad,
                             double inv_t, float* out, const double* accum, float* image, int n_sm, cudaStream_t st) {
-    // CTAs per (channel, pol): up to two CTAs per SM over the call, at least 2 antennas and 512 pixels each
-    int n_cl = 1;
-    while (n_cl < kAcMaxCluster && (long long)n_cp * n_cl < 2LL * n_sm && n_cl * 2 * 2 <= n_ant &&
-           n_pad * n_pad >= kAcThreads * n_cl * 2)
-        n_cl *= 2;
+    const int n_cl = autocorr_cluster(n_cp, n_ant, n_pad, lag_side, autocorr_smem_bytes(lag_side, n_pad, n_ant), n_sm);
     // at most autocorr_smem_bytes, which admitted the plan: the CTAs share out the powers
     const size_t smem = autocorr_smem_bytes(lag_side, n_pad, (n_ant + n_cl - 1) / n_cl);
     cudaError_t e = ensure_smem<autocorr_kernel>(smem);

@@ -1,5 +1,6 @@
 // Rules by which launches choose between kernel variants (host code; each with the measurements behind its line).
 #pragma once
+#include <cstddef>
 
 namespace epic {
 
@@ -27,6 +28,27 @@ inline int fx_planes_per_group(int n_cp, int n_pad, long long n_ent) {
         return g;
     }
     return n_cp >= 96 ? 32 : n_cp >= 40 ? 16 : n_cp >= 12 ? 8 : n_cp >= 6 ? 4 : n_cp >= 2 ? 2 : 1;
+}
+
+// Auto-correlation term: CTAs of a (channel, pol)'s cluster (kAcThreads = 512 threads each, at least two antennas and 512
+// pixels).  The CTAs share the antennas' sum and the pixels, but each does the first half of the transform, and past
+// what the SMs hold at once they come in waves: the least waves times (share done by each + rest / CTAs).  Clusters of
+// 4 and 8 leave some SMs of a GPC idle.  Measured (us a call of one sample; 1, 2, 4, 8 CTAs): 400 antennas of 15 x 15
+// cells, N_p = 512, one CTA an SM: 16 (channel, pol) 812, 487, 306, 339; 64: 1151, 741, 775, 963; 150: 1456, 1489, 1828,
+// 1962; 200: 2475, 2120, 2258, 2664; 331 antennas of 7 x 7 cells, N_p = 256, four an SM: 64: 165, 115, 103, 107; 150: 259,
+// 208, 223, 227; 400: 554, 538, 535, 579.
+inline int autocorr_cluster(long long n_cp, int n_ant, int n_pad, int lag_side, size_t smem, int n_sm) {
+    const long long fit = (long long)(228 * 1024 / (smem + 1024)), per_sm = fit < 1 ? 1 : fit > 4 ? 4 : fit;
+    // lags x pixels of a row in the first half of the transform; those of the whole image in the second
+    const double each = 0.05 + double(lag_side) / (lag_side + n_pad);
+    int best = 1;
+    double least = 0.0;
+    for (int n_cl = 1; n_cl <= 8 && (n_cl == 1 || (2 * n_cl <= n_ant && n_pad * n_pad >= 512 * n_cl)); n_cl *= 2) {
+        const long long held = n_sm * per_sm * (n_cl == 8 ? 28 : n_cl == 4 ? 36 : 38) / 38 / n_cl;
+        const double cost = double((n_cp + held - 1) / (held > 0 ? held : 1)) * (each + (1.0 - each) / n_cl);
+        if (n_cl == 1 || cost < least) best = n_cl, least = cost;
+    }
+    return best;
 }
 
 }  // namespace epic
