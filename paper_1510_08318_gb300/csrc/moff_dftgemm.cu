@@ -89,11 +89,17 @@ constexpr int NXW = 16;                   // transform warps: 4 per TMEM lane qu
 constexpr int NGW = 11;                   // gridding warps
 constexpr int NTH = 32 * (NXW + NGW + 1); // + the issuer's warp
 constexpr int NGT = 32 * NGW;             // gridding threads
-// Registers: 896 threads are launched with at most 72 each; the transform warps (32 FP32 sums and 32 columns
-// in flight) take 88, the others 48 (whole groups of four warps each): 16 x 88 + 12 x 48 <= 28 x 72.
-constexpr int kRegsTransform = 88, kRegsOther = 48;
-static_assert((NXW % 4) == 0 && ((NGW + 1) % 4) == 0 &&
-                  NXW * kRegsTransform + (NGW + 1) * kRegsOther <= (NXW + NGW + 1) * 72, "register split");
+// Registers: 896 threads are launched with at most 72 each, shared out by whole groups of four warps: the transform warps
+// (32 FP32 sums and 32 columns in flight) take 88 and the others 48, or 80 and 56 in the forms whose gridding warps need
+// more (two voltages a decode for XP) or whose transform warps need less (LP).  Measured (us): 262,144 images 3,675 and
+// 3,718; XP 32,768 images 565 and 549; LP 262,144 images 3,328 and 3,287.
+constexpr int regs_transform(bool xp, bool lp) { return xp || lp ? 80 : 88; }
+constexpr int regs_other(bool xp, bool lp) { return xp || lp ? 56 : 48; }
+constexpr bool split_fits(bool xp, bool lp) {
+    return NXW * regs_transform(xp, lp) + (NGW + 1) * regs_other(xp, lp) <= (NXW + NGW + 1) * 72;
+}
+static_assert((NXW % 4) == 0 && ((NGW + 1) % 4) == 0 && split_fits(false, false) && split_fits(true, false) &&
+                  split_fits(false, true), "register split");
 constexpr int WTAB = NP * NG;     // halves per [C ; S] table (hi or lo)
 constexpr int EIMG = 2 * NG * NG; // halves of one image's [Re ; Im] E^T rows
 constexpr int EPART = 2 * EIMG;   // halves of a pair's hi (or lo) E^T rows
@@ -153,6 +159,7 @@ __global__ void __launch_bounds__(NTH, 1) moff_dftgemm_kernel(const FwdArgs a, c
     using VT = typename Volt<VDT>::T;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     constexpr int NWT = LP ? 1 : 2, EBUF = ebuf(LP);
+    constexpr int kRegsTransform = regs_transform(XP, LP), kRegsOther = regs_other(XP, LP);
     __half* sW = reinterpret_cast<__half*>(smem_raw);                      // [NWT][WTAB]
     __half* sE = sW + NWT * WTAB;                                         // [2][EBUF]
     uint64_t* mbar = reinterpret_cast<uint64_t*>(sE + 2 * EBUF);          // [N_MBAR]
