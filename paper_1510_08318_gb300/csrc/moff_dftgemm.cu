@@ -317,7 +317,6 @@ __global__ void __launch_bounds__(NTH, 1) moff_dftgemm_kernel(const FwdArgs a, c
         int ecp = beg / T, et = beg - ecp * T, since = 0;   // the image being taken: (channel, pol), time; since a flush
         // after image `item` (local) is taken: add the sums into the accumulator where they must go
         auto taken = [&](int item) {
-            if (item >= n) return;
             ++since;
             const bool wrap = et + 1 == T;
             if (item + 1 == n || wrap || since == a.flush_every) {
@@ -342,10 +341,9 @@ __global__ void __launch_bounds__(NTH, 1) moff_dftgemm_kernel(const FwdArgs a, c
         };
 
         bool ok = true;
-        const int ni = 2 * np;                              // images, with the empty one of an odd last pair
 #pragma unroll 1
-        for (int i = -1; i < ni; ++i) {
-            if (i + 1 < ni) {
+        for (int i = -1; i < n; ++i) {
+            if (i + 1 < n) {
                 if (!(ok = warp_wait(MB_ST1 + ((i + 1) & 1), (i + 1) >> 1))) break;
                 fence_after();
                 split((i + 1) & 1);
@@ -655,7 +653,6 @@ __global__ void __launch_bounds__(NTH, 1) moff_dftgemm_kernel(const FwdArgs a, c
                 commit(mb(MB_F));
             };
             bool ok = true, issued = false;
-            const int ni = 2 * np;
             // stage 1 of image i, once its pair is gridded
             auto stage1 = [&](int i) -> bool {
                 const int j = i >> 1, img = i & 1;
@@ -674,15 +671,15 @@ __global__ void __launch_bounds__(NTH, 1) moff_dftgemm_kernel(const FwdArgs a, c
                 issued = true;
                 return true;
             };
-            ok = stage1(0) && stage1(1);
+            ok = stage1(0) && (n < 2 || stage1(1));   // an odd last pair has no second image
 #pragma unroll 1
-            for (int i = 0; ok && i < ni; ++i) {
+            for (int i = 0; ok && i < n; ++i) {
                 const int j = i >> 1, img = i & 1;
                 if (!(ok = wait(MB_XA + img, j))) break;
                 if (i > 0 && !(ok = wait(MB_FREE, i - 1))) break;
                 fence_after();
                 stage2(img);
-                if (i + 2 < ni) {
+                if (i + 2 < n) {
                     if (!(ok = wait(MB_F, i))) break;           // stage 2 has read the columns stage 1 overwrites
                     ok = stage1(i + 2);
                 }
