@@ -674,47 +674,46 @@ void pair_run_tables(int ng, int rows, int stride, int warps, int per, const std
                      const std::vector<float>& cwim, std::vector<int4>& run, std::vector<float2>& w, std::vector<float2>& wim,
                      std::vector<uint32_t>& key, std::vector<uint16_t>& empty) {
     constexpr int MAXW = 16;
-    const int NG = ng, NSLOT = rows * ng / 64;
+    const int NG = ng, NSLOT = rows * ng / 64, NPAIR = rows * ng / 2;
     struct Entry { int ant; float2 w, wi; };
-    struct Pair { int off; std::vector<Entry> e; };
     const float2 none = make_float2(0.f, 0.f);
     run.clear();
+    std::vector<Entry> all;                                  // the round's entries, pair by pair
+    std::vector<int> beg(NPAIR), cnt(NPAIR), cls[8], steps(NSLOT), order(NSLOT), mine[MAXW];
     for (int rb = 0; rb < ng / rows; ++rb) {
-        std::vector<Pair> pr(rows * NG / 2);
-        std::vector<std::vector<int>> cls(8);
-        for (int yp = 0; yp < rows / 2; ++yp)
-            for (int x = 0; x < NG; ++x) {
-                const int c = (rb * rows + 2 * yp) * NG + x;
-                Pair& p = pr[yp * NG + x];
-                p.off = 2 * yp * stride + x;
-                int i = cptr[c], j = cptr[c + NG];           // both in antenna order
-                while (i < cptr[c + 1] || j < cptr[c + NG + 1]) {
-                    const int ai = i < cptr[c + 1] ? cent[i].y : 1 << 30, aj = j < cptr[c + NG + 1] ? cent[j].y : 1 << 30;
-                    Entry e{std::min(ai, aj), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-                    if (ai == e.ant) {
-                        std::memcpy(&e.w.x, &cent[i].x, sizeof(float));
-                        e.wi.x = cwim[i++];
-                    }
-                    if (aj == e.ant) {
-                        std::memcpy(&e.w.y, &cent[j].x, sizeof(float));
-                        e.wi.y = cwim[j++];
-                    }
-                    p.e.push_back(e);
+        all.clear();
+        for (auto& c : cls) c.clear();
+        for (int q = 0; q < NPAIR; ++q) {
+            const int c = (rb * rows + 2 * (q / NG)) * NG + q % NG;
+            beg[q] = (int)all.size();
+            int i = cptr[c], j = cptr[c + NG];               // both in antenna order
+            while (i < cptr[c + 1] || j < cptr[c + NG + 1]) {
+                const int ai = i < cptr[c + 1] ? cent[i].y : 1 << 30, aj = j < cptr[c + NG + 1] ? cent[j].y : 1 << 30;
+                Entry e{std::min(ai, aj), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+                if (ai == e.ant) {
+                    std::memcpy(&e.w.x, &cent[i].x, sizeof(float));
+                    e.wi.x = cwim[i++];
                 }
-                cls[x & 7].push_back(yp * NG + x);
+                if (aj == e.ant) {
+                    std::memcpy(&e.w.y, &cent[j].x, sizeof(float));
+                    e.wi.y = cwim[j++];
+                }
+                all.push_back(e);
             }
-        for (auto& c : cls)
-            std::stable_sort(c.begin(), c.end(), [&](int u, int v) { return pr[u].e.size() > pr[v].e.size(); });
-        std::vector<int> steps(NSLOT, 0), order(NSLOT);
+            cnt[q] = (int)all.size() - beg[q];
+            cls[q & 7].push_back(q);                         // ng is a multiple of 8
+        }
+        for (auto& c : cls) std::stable_sort(c.begin(), c.end(), [&](int u, int v) { return cnt[u] > cnt[v]; });
         for (int r = 0; r < NSLOT; ++r) {
             order[r] = r;
-            for (auto& c : cls) steps[r] = std::max(steps[r], (int)pr[c[4 * r]].e.size());
+            steps[r] = 0;
+            for (auto& c : cls) steps[r] = std::max(steps[r], cnt[c[4 * r]]);
         }
         std::stable_sort(order.begin(), order.end(), [&](int u, int v) { return steps[u] > steps[v]; });
         // slots to the warps, heaviest first, each to the warp with the fewest steps (one for a slot that no antenna
         // reaches: its zeros are stored all the same)
-        std::vector<int> mine[MAXW];
         int load[MAXW] = {};
+        for (auto& v : mine) v.clear();
         for (int r : order) {
             const int wp = (int)(std::min_element(load, load + warps) - load);
             mine[wp].push_back(r);
@@ -723,46 +722,54 @@ void pair_run_tables(int ng, int rows, int stride, int warps, int per, const std
         for (int wp = 0; wp < warps; ++wp) {
             run.push_back(int4{(int)key.size(), 0, (int)empty.size(), 0});
             int4& me = run.back();
+            for (int r : mine[wp]) me.y += steps[r];
+            me.y = (me.y + kGridAhead - 1) / kGridAhead * kGridAhead;
+            size_t out = key.size();
+            // the steps past the last pair's keep zero weights, and an antenna (a run that is not empty has entries)
+            w.resize(out + 32 * (size_t)me.y, none);
+            wim.resize(w.size(), none);
+            key.resize(w.size(), me.y ? (uint32_t)cent[0].y : 0u);
             for (int r : mine[wp]) {
-                std::vector<Entry> rem[32];
+                Entry* rem[32];                              // a lane's remaining entries, in antenna order
+                int left[32];
                 uint32_t off[32];
                 for (int l = 0; l < 32; ++l) {
-                    const Pair& p = pr[cls[l & 7][4 * r + l / 8]];
-                    rem[l] = p.e;
-                    off[l] = (uint32_t)p.off;
-                    if (steps[r] == 0) empty.push_back((uint16_t)p.off);
+                    const int q = cls[l & 7][4 * r + l / 8];
+                    rem[l] = all.data() + beg[q];
+                    left[l] = cnt[q];
+                    off[l] = (uint32_t)(2 * (q / NG) * stride + q % NG);
+                    if (steps[r] == 0) empty.push_back((uint16_t)off[l]);
                 }
                 if (steps[r] == 0) ++me.w;
                 for (int k = 0; k < steps[r]; ++k) {
                     int pick[32], banks[4][16] = {}, some = -1;
                     for (int l = 0; l < 32; ++l) {
                         pick[l] = -1;
-                        if (rem[l].empty()) continue;
+                        if (left[l] == 0) continue;
                         // of the lane's remaining entries, one whose bank the lanes that load together use least at this step
                         pick[l] = 0;
-                        for (int j = 1; j < (int)rem[l].size(); ++j)
-                            if (banks[l / per][rem[l][j].ant & (per - 1)] < banks[l / per][rem[l][pick[l]].ant & (per - 1)]) pick[l] = j;
+                        int* use = banks[l / per];
+                        for (int j = 1; j < left[l]; ++j)
+                            if (use[rem[l][j].ant & (per - 1)] < use[rem[l][pick[l]].ant & (per - 1)]) pick[l] = j;
                         some = rem[l][pick[l]].ant;
-                        ++banks[l / per][some & (per - 1)];
+                        ++use[some & (per - 1)];
                     }
-                    for (int l = 0; l < 32; ++l) {
+                    for (int l = 0; l < 32; ++l, ++out) {
                         // past its list a lane gets zero weights and an antenna that another lane reads at this step
-                        const bool has = pick[l] >= 0;
-                        const Entry x = has ? rem[l][pick[l]] : Entry{some, none, none};
-                        w.push_back(x.w);
-                        wim.push_back(x.wi);
-                        key.push_back((uint32_t)x.ant | (k + 1 == steps[r] ? off[l] << 16 | kGridLast : 0u));
-                        if (has) rem[l].erase(rem[l].begin() + pick[l]);
+                        const uint32_t last = k + 1 == steps[r] ? off[l] << 16 | kGridLast : 0u;
+                        if (pick[l] < 0) {
+                            key[out] = (uint32_t)some | last;
+                            continue;
+                        }
+                        const Entry& x = rem[l][pick[l]];
+                        w[out] = x.w;
+                        wim[out] = x.wi;
+                        key[out] = (uint32_t)x.ant | last;
+                        std::memmove(rem[l] + pick[l], rem[l] + pick[l] + 1, (size_t)(left[l] - pick[l] - 1) * sizeof(Entry));
+                        --left[l];
                     }
                 }
-                me.y += steps[r];
             }
-            for (; me.y % kGridAhead != 0; ++me.y)
-                for (int l = 0; l < 32; ++l) {
-                    w.push_back(none);
-                    wim.push_back(none);
-                    key.push_back((uint32_t)cent[0].y);        // a run that is not empty has entries
-                }
         }
     }
 }
