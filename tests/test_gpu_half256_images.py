@@ -29,12 +29,12 @@ def epic():
 
 @pytest.mark.parametrize("n_ant, n_time, n_chan, n_pol, vdtype, complex_w, n_grid", [
     (1, 1, 76, 1, "c64", False, 128),
-    (2, 19, 2, 2, "f16", False, 101),
+    (2, 2, 19, 2, "f16", False, 101),
     (513, 3, 25, 1, "ci4", True, 128),
-    (60, 103, 3, 2, "f16", False, 128),
+    (60, 103, 5, 2, "f16", False, 128),
     (331, 608, 1, 1, "f16", False, 128),
     (1471, 15, 5, 1, "f16", False, 128),
-    (1025, 37, 4, 1, "c64", True, 90),
+    (1025, 152, 4, 1, "c64", True, 90),
 ])
 def test_image_power(epic, n_ant, n_time, n_chan, n_pol, vdtype, complex_w, n_grid):
     rng = np.random.default_rng([n_ant, n_time, n_chan])

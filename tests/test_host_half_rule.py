@@ -26,6 +26,23 @@ MEASURED = {
     (230400, 160, 1): (151.4, 370.6, 538.6, 450.1), (230400, 608, 1): (331.4, 1209.4, 1420.6, 1509.1),
     (297900, 76, 1): (84.4, 316.5, 211.2, 372.8), (297900, 304, 1): (212.2, 908.2, 804.7, 1094.6),
 }
+# the same forward, where sums begin and end in the middle of a worker's share
+MEASURED_FWD = {
+    (1525, 38, 4): (61.6, 57.6),
+    (1525, 14, 13): (82.1, 67.0),
+    (6775, 30, 4): (55.5, 52.5),
+    (6775, 22, 5): (70.4, 54.6),
+    (6775, 29, 5): (72.6, 61.8),
+    (6775, 20, 6): (70.4, 52.1),
+    (6775, 24, 6): (71.3, 53.5),
+    (6775, 76, 8): (153.1, 160.0),
+    (6775, 35, 13): (126.7, 123.5),
+    (6775, 7, 16): (71.4, 54.6),
+    (6775, 38, 16): (154.2, 161.3),
+    (9216, 152, 4): (145.1, 160.4),
+    (9216, 5, 24): (71.9, 55.6),
+    (74475, 20, 6): (84.4, 94.6),
+}
 # far enough apart that the halves have to be taken: where they save more than a fifth of the call
 CLEAR = 0.8
 
@@ -47,9 +64,10 @@ def rule(tmp_path_factory):
     exe = _compiled(tmp_path_factory, '    while (std::scanf("%lld %lld %lld", &e, &n, &c) == 3)\n'
                     '        std::printf("%d %d\\n", epic::half_pays_fwd(n, 152, double(e), c), '
                     'epic::half_pays_bwd(n, 152, double(e)));\n')
-    text = "".join("%d %d %d\n" % (e, t * c, c) for e, t, c in MEASURED)
+    cases = list(MEASURED) + list(MEASURED_FWD)
+    text = "".join("%d %d %d\n" % (e, t * c, c) for e, t, c in cases)
     out = subprocess.run([exe], input=text, capture_output=True, text=True, check=True).stdout.split()
-    return {k: (out[2 * i] == "1", out[2 * i + 1] == "1") for i, k in enumerate(MEASURED)}
+    return {k: (out[2 * i] == "1", out[2 * i + 1] == "1") for i, k in enumerate(cases)}
 
 
 @pytest.mark.parametrize("case", list(MEASURED), ids=lambda c: "x".join(map(str, c)))
@@ -60,6 +78,12 @@ def test_choice(rule, case):
             assert half
 
 
+@pytest.mark.parametrize("case", list(MEASURED_FWD), ids=lambda c: "x".join(map(str, c)))
+def test_choice_by_sums(rule, case):
+    h, c = MEASURED_FWD[case]
+    assert (h if rule[case][0] else c) <= 1.05 * c
+
+
 @pytest.mark.parametrize("items, n_ent, n_cp, cap, one_buffer, want", [
     (4096, 3000, 32, 0, 0, (1, 0)),          # no cap
     (4096, 3000, 32, 76, 0, (1, 76)),        # half images on 76 SMs
@@ -68,8 +92,8 @@ def test_choice(rule, case):
     (30, 3000, 1, 114, 0, (0, 28)),          # few images: clusters
     (30, 3000, 1, 3, 0, (0, 1)),
     (30, 3000, 1, 0, 0, (0, 0)),
-    (76, 3000, 4, 0, 0, (1, 0)),             # one wave of halves on 152 SMs, two on 76
-    (76, 3000, 4, 76, 0, (1, 76)),
+    (76, 3000, 19, 0, 0, (1, 0)),            # one wave of halves on 152 SMs, two on 76
+    (76, 3000, 19, 76, 0, (1, 76)),
     (77, 3000, 4, 76, 0, (0, 19)),           # three waves of halves and five of clusters
     (1 << 30, 3000, 32, 0, 0, (0, 0)),       # too many half images to number
 ])
