@@ -372,25 +372,18 @@ epic_status epic_create(epic_plan** plan, int n_ant, const double* pos_xy, const
     std::vector<float> awim;
     auto antenna_major = [&](int rows, int stride, std::vector<int>& aptr, std::vector<int2>& aent) {
         const int nq = NG / rows;
-        std::vector<std::vector<std::pair<int2, float>>> per_ant((size_t)nq * n_ant);
+        auto list = [&](const MapEntry& e) { return (size_t)(e.cell / NG / rows) * (n_ant + 1) + e.ant; };
+        aptr.assign((size_t)nq * (n_ant + 1) + 1, 0);
+        for (const MapEntry& e : m) ++aptr[list(e) + 1];
+        for (size_t i = 1; i < aptr.size(); ++i) aptr[i] += aptr[i - 1];
+        std::vector<int> at(aptr);                       // the next entry of each list
+        aptr.pop_back();
+        aent.resize(m.size());
+        awim.resize(m.size());
         for (const MapEntry& e : m) {
-            const int gy = e.cell / NG, gx = e.cell % NG;
-            const int q = gy / rows;
-            per_ant[(size_t)q * n_ant + e.ant].push_back({pack_entry(e.w, (gy - q * rows) * stride + gx), float(e.w.imag())});
-        }
-        aptr.assign((size_t)nq * (n_ant + 1), 0);
-        aent.reserve(m.size());
-        awim.clear();
-        awim.reserve(m.size());
-        for (int q = 0; q < nq; ++q) {
-            aptr[(size_t)q * (n_ant + 1)] = (int)aent.size();
-            for (int a = 0; a < n_ant; ++a) {
-                for (auto& pe : per_ant[(size_t)q * n_ant + a]) {
-                    aent.push_back(pe.first);
-                    awim.push_back(pe.second);
-                }
-                aptr[(size_t)q * (n_ant + 1) + a + 1] = (int)aent.size();
-            }
+            const int i = at[list(e)]++;
+            aent[i] = pack_entry(e.w, (e.cell / NG % rows) * stride + e.cell % NG);
+            awim[i] = float(e.w.imag());
         }
     };
     // the half-image kernels hold the whole grid: one block, its own row stride

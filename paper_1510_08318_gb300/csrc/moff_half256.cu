@@ -677,7 +677,22 @@ void pair_run_tables(int ng, int rows, int stride, int warps, int per, const std
     const int NG = ng, NSLOT = rows * ng / 64, NPAIR = rows * ng / 2;
     struct Entry { int ant; float2 w, wi; };
     const float2 none = make_float2(0.f, 0.f);
+    // by decreasing value, equal values in their order
+    std::vector<int> first, sorted;
+    auto by_decreasing = [&](std::vector<int>& v, const std::vector<int>& value) {
+        int most = 0;
+        for (int q : v) most = std::max(most, value[q]);
+        first.assign((size_t)most + 2, 0);
+        for (int q : v) ++first[most - value[q] + 1];
+        for (int i = 0; i <= most; ++i) first[i + 1] += first[i];
+        sorted.resize(v.size());
+        for (int q : v) sorted[first[most - value[q]]++] = q;
+        v.swap(sorted);
+    };
     run.clear();
+    w.reserve(w.size() + cent.size());
+    wim.reserve(wim.size() + cent.size());
+    key.reserve(key.size() + cent.size());
     std::vector<Entry> all;                                  // the round's entries, pair by pair
     std::vector<int> beg(NPAIR), cnt(NPAIR), cls[8], steps(NSLOT), order(NSLOT), mine[MAXW];
     for (int rb = 0; rb < ng / rows; ++rb) {
@@ -703,13 +718,13 @@ void pair_run_tables(int ng, int rows, int stride, int warps, int per, const std
             cnt[q] = (int)all.size() - beg[q];
             cls[q & 7].push_back(q);                         // ng is a multiple of 8
         }
-        for (auto& c : cls) std::stable_sort(c.begin(), c.end(), [&](int u, int v) { return cnt[u] > cnt[v]; });
+        for (auto& c : cls) by_decreasing(c, cnt);
         for (int r = 0; r < NSLOT; ++r) {
             order[r] = r;
             steps[r] = 0;
             for (auto& c : cls) steps[r] = std::max(steps[r], cnt[c[4 * r]]);
         }
-        std::stable_sort(order.begin(), order.end(), [&](int u, int v) { return steps[u] > steps[v]; });
+        by_decreasing(order, steps);
         // slots to the warps, heaviest first, each to the warp with the fewest steps (one for a slot that no antenna
         // reaches: its zeros are stored all the same)
         int load[MAXW] = {};
