@@ -217,7 +217,7 @@ struct DgGather {
     // (read by the FP16-gridding form); nullptr otherwise
     const uint32_t* wpk = nullptr;
 };
-// N_p = 128: the size that decides how many antennas the form accepts (a launch needs at most this); lp:
+// N_p = 128: the size that decides how many antennas the form accepts (see there); lp:
 // the reduced-precision form (FP16 operands and one product per real product)
 size_t dftgemm_smem_bytes(int n_ant, bool xpol = false, bool lp = false);
 void dftgemm_tables(std::vector<uint16_t>& out);

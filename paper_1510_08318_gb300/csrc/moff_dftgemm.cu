@@ -709,10 +709,15 @@ __global__ void __launch_bounds__(NTH, 1) moff_dftgemm_kernel(const FwdArgs a, c
 
 }  // namespace dg
 
-// The antennas the form accepts follow from this size against the device's limit; what the kernel asks
-// for with one voltage buffer (dg::smem_fixed + 20 bytes per antenna) is below it for every count accepted.
+// The antennas the form accepts follow from this size against the device's limit: 2,448 of 232,448 bytes, 1,904 for
+// cross-polarisation.  It is the documented limit, not the kernel's need: with one voltage buffer that is dg::smem_fixed
+// (192 bytes more than here) and 20 bytes an antenna (12 for LP), so it fits wherever this does from 24 antennas on, and
+// under 24 antennas on any device that takes 24.
 size_t dftgemm_smem_bytes(int n_ant, bool xpol, bool lp) {
-    return (lp ? 81984 : 163904) + (size_t)n_ant * ((xpol ? 36 : 28) - (lp ? 8 : 0));
+    constexpr size_t kFull = 163904, kLp = 81984;
+    static_assert(dg::smem_fixed(false) + 24 * dg::ant_bytes(false, 1) <= kFull + 24 * 28 &&
+                      dg::smem_fixed(true) + 24 * dg::ant_bytes(true, 1) <= kLp + 24 * 20, "need within the limit");
+    return (lp ? kLp : kFull) + (size_t)n_ant * ((xpol ? 36 : 28) - (lp ? 8 : 0));
 }
 
 // Operand tables for N_p = 128: two [128][64] K-major FP16 tables (hi parts, then lo parts) of the rows
@@ -854,7 +859,7 @@ bool dftgemm_gather_tables_ng(int ng, int n_warps, const std::vector<int>& cptr,
     return true;
 }
 
-// The builder above on the 64 x 64 grid with 16 warps (one weight per entry).
+// The builder above on the 64 x 64 grid with 16 warps (one weight per entry): the checker of its slots calls it.
 bool dftgemm_gather_tables(const std::vector<int>& cptr, const std::vector<int2>& cent, const std::vector<float>& cwim,
                            std::vector<int2>& lane, std::vector<int>& base, std::vector<float>& wre,
                            std::vector<float>& wim, std::vector<uint16_t>& ant) {
