@@ -57,6 +57,8 @@ DG_LP_FLOP_PER_IMAGE = DG_ALG_FLOP_PER_IMAGE / 2
 DG_TENSOR_ACTIVE_NCU = 0.519
 # standalone gridder: 479.8 MB per capture launch (1,024 of the 16,384 units), scaled x16
 GRID_TRAFFIC_BYTES = 7.677e9
+# forms of the cross-polarisation mode (the FP16-gridding one exists at N_p = 256 only, without these products)
+XPOL_FORMS = (("fp32_fft", "fft"), ("fp16x3_dftgemm", "dftgemm"))
 MEASURED_PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 try:
     with open(MEASURED_PEAKS) as _f:
@@ -764,8 +766,7 @@ def run_xpol(args):
         return max_over_ranks([sum(a.elapsed_time(b) for a, b in ev) / args.steps], world, dev)[0], clk
 
     forms = {}
-    for name, xf in (("fp32_fft", "fft"), ("fp16x3_dftgemm", "dftgemm"),
-                     ("fp16grid_fp16x3_dftgemm", "dftgemm_fp16grid")):
+    for name, xf in XPOL_FORMS:
         plan.set_transform(xf)
         for _ in range(max(args.warmup, 3)):
             step()
